@@ -143,7 +143,6 @@ struct Work {
     // output and the down projection, and the chunk partials [kWideBlocks][max_chunks][8][H][hd+2] of the untiled attention
     // (128 rows at most).  Every writer waits for its predecessor, which has consumed what was there.
     float* pf_part;
-    size_t pf_part_floats;
     size_t pf_attn_stride;                     // floats per block of chunk partials
     void* k_cache;         // [L][n_pages][page][kvd]
     void* v_cache;
@@ -200,16 +199,12 @@ static size_t carve(const Dims& D, char* base, bool with_state, Work* w) {
             c.take(W.pf_act_f, es * 2 * rows * D.F);
             c.take(W.pf_q, sizeof(float) * rows * D.qd);
             W.pf_attn_stride = (size_t)max_chunks * kMaxW * D.H * (D.hd + 2);
-            // room for 8 splits of one tile; with more tiles, for the fewest splits their sums are allowed to have
-            const size_t tiles = rows / kTileRowsPf, ntot = (size_t)D.qd + 2 * D.kvd;
-            auto part = [&](int K, size_t n) {
-                const size_t least = tiles * (size_t)tc_wide_min_splits(K);
-                return (size_t)kTileRowsPf * n * (least > (size_t)kMaxSplit ? least : (size_t)kMaxSplit);
-            };
-            W.pf_part_floats = (size_t)kWideBlocks * W.pf_attn_stride;
-            for (size_t n : {part(D.d, ntot), part(D.qd, (size_t)D.d), part(D.F, (size_t)D.d)})
-                if (n > W.pf_part_floats) W.pf_part_floats = n;
-            c.take(W.pf_part, sizeof(float) * W.pf_part_floats);
+            const int tiles = (int)rows / kTileRowsPf;
+            size_t floats = (size_t)kWideBlocks * W.pf_attn_stride;
+            for (size_t n : {tc_wide_partial_rows(D.d, tiles) * (D.qd + 2 * D.kvd), tc_wide_partial_rows(D.qd, tiles) * D.d,
+                             tc_wide_partial_rows(D.F, tiles) * D.d})
+                if (n > floats) floats = n;
+            c.take(W.pf_part, sizeof(float) * floats);
         }
         c.take(W.rope_tab, sizeof(float2) * (size_t)D.n_pages * D.page * (D.hd / 2));
         size_t kv = es * (size_t)D.L * D.n_pages * D.page * D.kvd;
@@ -256,7 +251,6 @@ static int gemm(Exec& e, const void* const* W, const int* N, int n_mats, int K, 
                 void* swiglu_out = nullptr, const NextGemm& next = NextGemm(), int nb = 1) {
     GemmArgs a{};
     a.nb = nb;
-    a.out_floats = nb > 1 ? e.W.pf_part_floats : 0;
     a.swiglu_out = swiglu_out;
     a.next_W[0] = next.W[0]; a.next_W[1] = next.W[1]; a.next_rows = next.rows; a.next_K = next.K; a.next_act = next.act;
     int tot = 0;

@@ -865,11 +865,25 @@ static int wide_min_splits(int KB) {
     const int s = (KB + kWideMaxChain - 1) / kWideMaxChain;
     return s < kMaxSplit ? s : kMaxSplit;   // consumers sum at most kMaxSplit partials
 }
-int tc_wide_min_splits(int K) { return wide_min_splits((K + kBK - 1) / kBK); }
-static void choose_split_cta_pair(const int* n_rows, int n_mats, int KB, int max_split, int G, int* R_out, int* S_out, int n_tiles = 1) {
+// Most k splits of a wide GEMM: 8 for one tile; with more, what 8 splits of one tile or the fewest allowed splits of all of
+// them write (33 MB of partials for 512 rows of the 7B output projection: beside the weights they stay in L2).  A function
+// of k and the number of tiles only: the order of a prompt's sums must not depend on how long its context may grow.
+static int wide_max_splits(int KB, int n_tiles) {
+    const int least = wide_min_splits(KB);
+    return n_tiles * least > kMaxSplit ? least : kMaxSplit / n_tiles;
+}
+size_t tc_wide_partial_rows(int K, int n_tiles) {
+    size_t most = 0;
+    for (int t = 1; t <= n_tiles; ++t) {
+        const size_t rows = (size_t)t * kWideBlocks * kMaxW * wide_max_splits((K + kBK - 1) / kBK, t);
+        if (rows > most) most = rows;
+    }
+    return most;
+}
+static void choose_split_cta_pair(const int* n_rows, int n_mats, int KB, int G, int* R_out, int* S_out, int n_tiles = 1) {
     double best = 1e300;
     int bR = 128, bS = 1;
-    for (int S = n_tiles > 1 ? wide_min_splits(KB) : 1; S <= max_split && S <= KB; ++S)
+    for (int S = n_tiles > 1 ? wide_min_splits(KB) : 1; S <= wide_max_splits(KB, n_tiles) && S <= KB; ++S)
         for (int R = 128; R >= 8; R -= 8) {
             long long chunks = 0;
             for (int j = 0; j < n_mats; ++j) chunks += (n_rows[j] + 2 * R - 1) / (2 * R);
@@ -909,7 +923,7 @@ static int max_pair_clusters();
 // nb: blocks of 8 activation rows.  cta_pair: plan for k_tc_pair (a work item is a slab of 2 R rows for a cluster of two
 // CTAs and one of the nb / kWideBlocks tiles of 128 activation rows)
 static TcPlan* get_plan(TcPlanCache* cache, const void* const* W, const int* n_end, int n_mats, int K, const void* act,
-                        bool head, bool pair = false, int nb = 1, bool cta_pair = false, size_t out_floats = 0) {
+                        bool head, bool pair = false, int nb = 1, bool cta_pair = false) {
     std::vector<uint64_t> key;
     for (int j = 0; j < n_mats; ++j) { key.push_back((uint64_t)(uintptr_t)W[j]); key.push_back((uint64_t)n_end[j]); }
     key.push_back((uint64_t)K);
@@ -948,10 +962,8 @@ static TcPlan* get_plan(TcPlanCache* cache, const void* const* W, const int* n_e
         chunks = (p.n_rows[0] + p.pair_half - 1) / p.pair_half;
         for (int j = 0; j < 3; ++j) p.chunk_end[j] = chunks;
     } else {
-        if (cta_pair) {
-            const size_t room = out_floats / ((size_t)p.n_tiles * kWideBlocks * kMaxW * prev);   // splits the partials have room for
-            choose_split_cta_pair(p.n_rows, n_mats, p.KB, room < (size_t)kMaxSplit ? (int)room : kMaxSplit, G, &p.R, &p.S, p.n_tiles);
-        } else choose_split(p.n_rows, n_mats, p.KB, head ? 1 : kMaxSplit, G, &p.R, &p.S);
+        if (cta_pair) choose_split_cta_pair(p.n_rows, n_mats, p.KB, G, &p.R, &p.S, p.n_tiles);
+        else choose_split(p.n_rows, n_mats, p.KB, head ? 1 : kMaxSplit, G, &p.R, &p.S);
         for (int j = 0; j < 3; ++j) {
             if (j < n_mats) chunks += (p.n_rows[j] + per_item * p.R - 1) / (per_item * p.R);
             p.chunk_end[j] = chunks;
@@ -979,7 +991,7 @@ bool tc_plan_query(int mode, const int* n_rows, int n_mats, int K, int units, in
         *R = h; *S = 1; *n_items = (n_rows[0] + h - 1) / h;
         return true;
     }
-    if (mode == 2) choose_split_cta_pair(n_rows, n_mats, KB, kMaxSplit, units, R, S);
+    if (mode == 2) choose_split_cta_pair(n_rows, n_mats, KB, units, R, S);
     else choose_split(n_rows, n_mats, KB, kMaxSplit, units, R, S);
     const int per = mode == 2 ? 2 : 1;
     int chunks = 0;
@@ -1101,7 +1113,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& a, TcPlanCache* cache, unsig
     if (cta_pair) nb = (nb + kWideBlocks - 1) / kWideBlocks * kWideBlocks;
     else nb = nb <= 2 ? nb : nb <= 4 ? 4 : kWideBlocks;
     if (a.nb > nb || nb * kMaxW > kMaxWideRows) return -1;
-    TcPlan* pl = get_plan(cache, a.W, a.n_end, a.n_mats, a.K, a.act, false, pair, nb, cta_pair, a.out_floats);
+    TcPlan* pl = get_plan(cache, a.W, a.n_end, a.n_mats, a.K, a.act, false, pair, nb, cta_pair);
     if (!pl) return -1;
     TcParams p = pl->p;
     p.out = a.out; p.n_total = a.n_total; p.r0 = a.r0; p.m = a.m; p.status = status;

@@ -31,8 +31,8 @@ bool tc_set_split_penalty(int per_mille);
 // wide passes (GemmArgs::nb > 1): true (default) = clusters of two CTAs sharing one activation tile (cta_group::2),
 // false = one CTA per work item
 void tc_set_wide_cta_pairs(bool on);
-// fewest k splits of a wide GEMM over k = K (see kWideMaxChain)
-int tc_wide_min_splits(int K);
+// rows of fp32 partials (as wide as the output) that a wide GEMM over k = K of up to n_tiles 128-row tiles leaves at most
+size_t tc_wide_partial_rows(int K, int n_tiles);
 int tc_wide_rows();   // most prompt rows one wide pass can take under that setting on the current device
 // the work decomposition for `units` CTAs (modes 0, 1: 8-row kernel, its gate/up form) or clusters (modes 2, 3: CTA-pair
 // kernel, its gate/up form): rows per CTA (gate/up: columns per item), k splits, work items.  Host arithmetic only.

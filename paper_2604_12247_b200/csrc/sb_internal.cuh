@@ -384,7 +384,6 @@ struct GemmArgs {          // out[s][row][n] = sum_k act[row][k] * W[n][k]   for
     // of 128-row tiles).  act is then [nb][16][K] (block b = rows 8b .. 8b+7: high halves, low halves), out is [nb][n_split][8][n_total],
     // swiglu_out [nb][16][n_end[0]], and r0 / m count rows over all blocks.  0 or 1: one block.
     int nb;
-    size_t out_floats;     // wide mode: floats that out has room for (bounds the k splits)
 };
 
 struct HeadArgs {          // exit-confidence / final-head kernel

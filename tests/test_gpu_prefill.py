@@ -132,3 +132,20 @@ def test_wide_prefill_at_the_bench_shape_matches_narrow_first_token_and_tokens()
     assert out["stats"].us_prefill < 0.6 * out_n["stats"].us_prefill
     assert np.array_equal(out["tokens"], out_n["tokens"])
     ctx.close()
+
+
+# three and four 128-row tiles at the 7B widths, whose GEMMs are split along k: the order of a prompt's sums is the prompt's
+# alone, whatever room the context has beside it (the chunk partials of 8192 positions are the larger part of its scratch)
+@pytest.mark.parametrize("n_prompt", [300, 512])
+def test_wide_prefill_does_not_depend_on_the_capacity_of_the_context(n_prompt):
+    shape = inputs.scaled(inputs.LLAMA2_7B, name="7b-2-layers", n_layers=2, vocab=2048)
+    w = inputs.make_weights(shape, 6, device="cuda")
+    pr = inputs.make_prompt(shape, n_prompt, 6).numpy()
+    got = []
+    for max_seq in (540, 8192):
+        ctx = binding.Context(shape, w, max_seq, kv_page=64)
+        got.append(_hidden_after_prefill(ctx, pr, shape.n_layers))
+        ctx.close()
+    assert got[0][0] == got[1][0]
+    for a, b in zip(got[0][1], got[1][1]):
+        assert np.array_equal(a, b)
