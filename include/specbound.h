@@ -328,10 +328,12 @@ int sb_set_default_option(int32_t key, int32_t value);
  * steps and of the unified pass; Section 4.3: prefill).  Host arithmetic only: no device is touched, nothing is launched;
  * meant for tests and for sizing studies.
  *   mode 0: the 8-row kernel on `units` CTAs; 1: its gate/up form (n_rows[0] = FFN width, n_mats = 1);
- *   mode 2: the 128-row kernel on `units` clusters of two CTAs; 3: its gate/up form.
+ *   mode 2: the kernel of the wide prefill passes on `units` clusters of two CTAs, for one tile of 128 rows; 3: its gate/up
+ *   form in items of one accumulator (up to 128 columns).  mode 2 + 256 t, 3 + 256 t, t = 1..4: as the GEMMs of a pass of
+ *   t tiles run it; a gate/up item of one tile may then have up to 256 columns, in two accumulators.
  *   n_rows[n_mats] (1..3 matrices that share k and the activation operand, HOST array), k = inner dimension.
  * Out (HOST): rows_per_cta = weight rows a CTA stages per work item (gate/up: FFN columns per item), k_splits, n_items =
- * slabs x splits.  Returns SB_ERR_ARG for null pointers, mode outside 0..3, n_mats outside 1..3 or non-positive sizes. */
+ * slabs x splits (x tiles).  Returns SB_ERR_ARG for null pointers, any other mode, n_mats outside 1..3 or non-positive sizes. */
 int sb_plan_gemm(int32_t mode, const int32_t* n_rows, int32_t n_mats, int32_t k, int32_t units, int32_t* rows_per_cta,
                  int32_t* k_splits, int32_t* n_items);
 

@@ -919,6 +919,23 @@ static int choose_one_round_cols(int n_rows, int G, int two_round_cols) {
     return h <= rounds * (two_round_cols > g_pair_floor_rows ? two_round_cols : g_pair_floor_rows) ? h : 0;
 }
 
+// Work decomposition of the CTA-pair kernel, for the launches (get_plan) and for tc_plan_query alike: rows a CTA stages per
+// item (gate/up: FFN columns of the item), k splits, parts of an item (2: choose_one_round_cols), slabs
+struct PairPlan { int R, S, n_sub, chunks; };
+static PairPlan plan_cta_pair(bool gate_up, const int* n_rows, int n_mats, int KB, int G, int n_tiles) {
+    PairPlan d{0, 1, 1, 0};
+    if (gate_up) {
+        d.R = choose_cols_cta_pair(n_rows[0], G, n_tiles);
+        const int one_round = n_tiles == 1 ? choose_one_round_cols(n_rows[0], G, d.R) : 0;
+        if (one_round > 0) { d.R = one_round; d.n_sub = 2; }
+        d.chunks = (n_rows[0] + d.R - 1) / d.R;
+        return d;
+    }
+    choose_split_cta_pair(n_rows, n_mats, KB, G, &d.R, &d.S, n_tiles);
+    for (int j = 0; j < n_mats; ++j) d.chunks += (n_rows[j] + 2 * d.R - 1) / (2 * d.R);
+    return d;
+}
+
 static int max_pair_clusters();
 // nb: blocks of 8 activation rows.  cta_pair: plan for k_tc_pair (a work item is a slab of 2 R rows for a cluster of two
 // CTAs and one of the nb / kWideBlocks tiles of 128 activation rows)
@@ -946,14 +963,15 @@ static TcPlan* get_plan(TcPlanCache* cache, const void* const* W, const int* n_e
     for (int j = 0; j < n_mats; ++j) { p.n_rows[j] = n_end[j] - prev; p.n_off[j] = prev; prev = n_end[j]; }
     int chunks = 0;
     const int per_item = cta_pair ? 2 : 1;   // CTAs that share a work item
+    PairPlan pp{};
+    if (cta_pair) {
+        pp = plan_cta_pair(pair, p.n_rows, n_mats, p.KB, G, p.n_tiles);
+        p.R = pp.R; p.S = pp.S; p.n_sub = pp.n_sub;
+    }
     if (pair && cta_pair) {
-        p.pair_half = choose_cols_cta_pair(p.n_rows[0], G, p.n_tiles);
-        const int one_round = p.n_tiles == 1 ? choose_one_round_cols(p.n_rows[0], G, p.pair_half) : 0;
-        if (one_round > 0) { p.pair_half = one_round; p.n_sub = 2; }
+        p.pair_half = p.R;
         p.stages = pair_stages(p.pair_half);
-        p.R = p.pair_half;
-        p.S = 1;
-        chunks = (p.n_rows[0] + p.pair_half - 1) / p.pair_half;
+        chunks = pp.chunks;
         for (int j = 0; j < 3; ++j) p.chunk_end[j] = chunks;
     } else if (pair) {
         p.pair_half = choose_pair_half(p.n_rows[0], G);
@@ -962,8 +980,7 @@ static TcPlan* get_plan(TcPlanCache* cache, const void* const* W, const int* n_e
         chunks = (p.n_rows[0] + p.pair_half - 1) / p.pair_half;
         for (int j = 0; j < 3; ++j) p.chunk_end[j] = chunks;
     } else {
-        if (cta_pair) choose_split_cta_pair(p.n_rows, n_mats, p.KB, G, &p.R, &p.S, p.n_tiles);
-        else choose_split(p.n_rows, n_mats, p.KB, head ? 1 : kMaxSplit, G, &p.R, &p.S);
+        if (!cta_pair) choose_split(p.n_rows, n_mats, p.KB, head ? 1 : kMaxSplit, G, &p.R, &p.S);
         for (int j = 0; j < 3; ++j) {
             if (j < n_mats) chunks += (p.n_rows[j] + per_item * p.R - 1) / (per_item * p.R);
             p.chunk_end[j] = chunks;
@@ -979,23 +996,30 @@ static TcPlan* get_plan(TcPlanCache* cache, const void* const* W, const int* n_e
     return pl;
 }
 
-// The decomposition the launches use, for a given number of CTAs (8-row kernel) or clusters (CTA-pair kernel): host
-// arithmetic only.  mode 0: 8-row kernel, 1: its gate/up form, 2: 128-row CTA-pair kernel, 3: its gate/up form.
+// The work decomposition for a given number of CTAs (8-row kernel) or clusters (CTA-pair kernel): host arithmetic only.
+// mode 0: 8-row kernel, 1: its gate/up form, 2: CTA-pair kernel on one tile of 128 rows, 3: its gate/up form in items of one
+// accumulator.  mode 2 or 3 plus 256 * t: what the launches of a pass of t tiles use (one tile's gate/up may be in two parts).
 bool tc_plan_query(int mode, const int* n_rows, int n_mats, int K, int units, int* R, int* S, int* n_items) {
-    if (mode < 0 || mode > 3 || !n_rows || n_mats < 1 || n_mats > 3 || K < 1 || units < 1) return false;
+    const int n_tiles = mode >> 8, form = mode & 255;
+    if (mode < 0 || form > 3 || n_tiles > kMaxWideRows / (kWideBlocks * kMaxW) || (n_tiles > 0 && form < 2)) return false;
+    if (!n_rows || n_mats < 1 || n_mats > 3 || K < 1 || units < 1) return false;
     for (int j = 0; j < n_mats; ++j)
         if (n_rows[j] < 1) return false;
     const int KB = (K + kBK - 1) / kBK;
-    if (mode == 1 || mode == 3) {
-        const int h = mode == 3 ? choose_cols_cta_pair(n_rows[0], units) : choose_pair_half(n_rows[0], units);
+    if (n_tiles > 0 || form == 2) {
+        const int tiles = n_tiles > 0 ? n_tiles : 1;
+        const PairPlan d = plan_cta_pair(form == 3, n_rows, n_mats, KB, units, tiles);
+        *R = d.R; *S = d.S; *n_items = d.chunks * d.S * tiles;
+        return true;
+    }
+    if (form == 1 || form == 3) {
+        const int h = form == 3 ? choose_cols_cta_pair(n_rows[0], units) : choose_pair_half(n_rows[0], units);
         *R = h; *S = 1; *n_items = (n_rows[0] + h - 1) / h;
         return true;
     }
-    if (mode == 2) choose_split_cta_pair(n_rows, n_mats, KB, units, R, S);
-    else choose_split(n_rows, n_mats, KB, kMaxSplit, units, R, S);
-    const int per = mode == 2 ? 2 : 1;
+    choose_split(n_rows, n_mats, KB, kMaxSplit, units, R, S);
     int chunks = 0;
-    for (int j = 0; j < n_mats; ++j) chunks += (n_rows[j] + per * *R - 1) / (per * *R);
+    for (int j = 0; j < n_mats; ++j) chunks += (n_rows[j] + *R - 1) / *R;
     *n_items = chunks * *S;
     return true;
 }

@@ -35,7 +35,8 @@ void tc_set_wide_cta_pairs(bool on);
 size_t tc_wide_partial_rows(int K, int n_tiles);
 int tc_wide_rows();   // most prompt rows one wide pass can take under that setting on the current device
 // the work decomposition for `units` CTAs (modes 0, 1: 8-row kernel, its gate/up form) or clusters (modes 2, 3: CTA-pair
-// kernel, its gate/up form): rows per CTA (gate/up: columns per item), k splits, work items.  Host arithmetic only.
+// kernel on one tile, its gate/up form in items of one accumulator; + 256 * t: as the launches of a pass of t tiles have it):
+// rows per CTA (gate/up: columns per item), k splits, work items.  Host arithmetic only.
 bool tc_plan_query(int mode, const int* n_rows, int n_mats, int K, int units, int* R, int* S, int* n_items);
 // returns the number of split-K partials written to a.out, or -1 if no TMA descriptor could be made
 int launch_gemm_tc(cudaStream_t st, const GemmArgs& a, TcPlanCache* cache, unsigned int* status);

@@ -53,3 +53,48 @@ def test_plan_query_rejects_bad_arguments():
         binding.plan_gemm(2, [4096], 0, 74)
     with pytest.raises(binding.SBError):
         binding.plan_gemm(2, [4096], 4096, 0)
+
+
+# the decompositions the wide prefill passes launch, one to four tiles of 128 rows: what the kernel can run, the bound on the
+# length of a sum, partials that fit their buffer, and everything covered
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: s.name)
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4])
+@pytest.mark.parametrize("units", [66, 72, 74])
+def test_wide_pass_plans(shape, tiles, units):
+    for name, (n_rows, k) in _gemms(shape).items():
+        R, S, items = binding.plan_gemm(2 + 256 * tiles, n_rows, k, units)
+        kb = math.ceil(k / 64)
+        assert R % 8 == 0 and 8 <= R <= 128 and 1 <= S <= min(8, kb), (name, R, S)
+        assert items == sum(math.ceil(n / (2 * R)) for n in n_rows) * S * tiles
+        if tiles > 1:
+            assert math.ceil(kb / S) <= 45, (name, S)                  # k blocks that one accumulator takes in
+            least = math.ceil(kb / 45)
+            assert S * tiles <= max(8, least * tiles), (name, S)       # rows of partials the workspace holds
+        else:
+            assert (R, S, items) == binding.plan_gemm(2, n_rows, k, units)
+        busiest = math.ceil(items / units) * 2 * R * math.ceil(kb / S)
+        if shape.name != "small":
+            assert busiest <= 1.6 * sum(n_rows) * kb * tiles / units, (name, R, S, items)
+
+
+@pytest.mark.parametrize("d_ffn", [1408, 1416, 9472, 9480, 11008, 11016, 13824, 14336, 18944, 18952, 28672])
+@pytest.mark.parametrize("tiles", [1, 2, 4])
+@pytest.mark.parametrize("units", [66, 72, 74])
+def test_wide_pass_gate_up_plans(d_ffn, tiles, units):
+    h, S, items = binding.plan_gemm(3 + 256 * tiles, [d_ffn], 4096, units)
+    assert S == 1 and h % 8 == 0 and 8 <= h <= 256
+    assert items == math.ceil(d_ffn / h) * tiles
+    if h > 128:                                       # two accumulators: one round of one tile, halves the MMA can take
+        assert tiles == 1 and h % 16 == 0 and items <= units
+        stage = h * 128 + 16384                       # bytes of a pipeline stage; at least one per producer fits
+        assert 4 * stage + 1280 <= 225 * 1024
+    else:                                             # and where one round of two parts is the shorter one, it is taken
+        rounds = math.ceil(math.ceil(d_ffn / h) / units)
+        one = math.ceil(math.ceil(d_ffn / units) / 16) * 16
+        assert tiles > 1 or rounds == 1 or one > 256 or one > rounds * max(h, 96)
+
+
+def test_plan_query_rejects_bad_tile_counts():
+    for mode in (256, 257, 2 + 256 * 5, 4 + 256, -254):
+        with pytest.raises(binding.SBError):
+            binding.plan_gemm(mode, [4096], 4096, 74)
