@@ -110,6 +110,34 @@ def test_nucleus_sampling_at_the_edges_of_its_instances(vocab, ties):
     assert _compare_with_oracle_samples(z.numpy(), 1.0, 5, 9, tok, edge_tol=1e-9, top_p=top_p) == 0
 
 
+# nearly flat rows, whose tokens lie close together beside (or without) a maximum far above them: more tokens in the deciding
+# bucket than the list holds, with one key (taken as it is), two neighbouring keys, a range of keys of one exponent (two digits
+# of the radix select) and one through zero (three)
+@pytest.mark.parametrize("vocab", [32000, 262144])
+@pytest.mark.parametrize("top_p", [0.3, 0.9])
+def test_nucleus_sampling_of_nearly_flat_rows(vocab, top_p):
+    g = torch.Generator().manual_seed(vocab)
+    flat = torch.randn(8, vocab, generator=g)
+    z = torch.empty(8, vocab)
+    z[0] = 0.1 * flat[0]
+    z[1] = 1e-6 * flat[1]
+    z[2] = 0.01 * flat[2] + 1.0
+    z[3] = 0.5
+    z[4] = torch.where(flat[4] > 0, torch.tensor(0.5), torch.nextafter(torch.tensor(0.5), torch.tensor(1.0)))
+    z[5] = 1e-4 * flat[5]
+    z[6] = -0.003 * flat[6].abs() - 2.0
+    z[7] = torch.round(256 * flat[7]) / 256           # as if out of a 16-bit head
+    at = torch.randperm(vocab, generator=g)[:8]
+    for j in (2, 3, 4, 5, 6):
+        z[j, at[j]] += 6.0
+    top_p = f32(top_p)
+    tok = binding.k_sample(z.cuda(), 1.0, 8, 21, top_p=top_p).cpu().numpy()
+    for j in range(8):
+        zs = oracle.nucleus_threshold(z[j].double().numpy(), 1.0, top_p)
+        assert float(z[j, tok[j]]) >= zs, (j, tok[j], zs)
+    assert _compare_with_oracle_samples(z.numpy(), 1.0, 8, 21, tok, edge_tol=1e-9, top_p=top_p) == 0
+
+
 def test_sampling_kernel_frequencies_follow_softmax():
     g = torch.Generator().manual_seed(1)
     V, T, N = 200, 0.9, 4000
