@@ -439,7 +439,7 @@ static void head(Exec& e, const void* lm_head, int r0, int m, float tau, float t
         if (!launch_head_tc(e.st, a, e.plans, e.W.status)) e.err = SB_ERR_CUDA;
         return;
     }
-    SB_T(e, launch_head_simt<T>(e.st, a, 148 * 4));
+    SB_T(e, launch_head_simt<T>(e.st, a));
 }
 
 }  // namespace sb

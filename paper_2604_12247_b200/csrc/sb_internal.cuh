@@ -479,6 +479,6 @@ void launch_init_pages(cudaStream_t st, int* page_table, int n_pages);
 
 // ---- launchers (gemm_simt.cu) ----
 template <typename T> void launch_gemm_simt(cudaStream_t st, const GemmArgs& a);
-template <typename T> void launch_head_simt(cudaStream_t st, const HeadArgs& a, int n_ctas);
+template <typename T> void launch_head_simt(cudaStream_t st, const HeadArgs& a);
 
 }  // namespace sb

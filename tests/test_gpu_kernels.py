@@ -263,6 +263,36 @@ def test_cuda_core_layer_with_and_without_the_swiglu_launch(d_model, d_ffn):
         assert np.abs(fused[0] - want).max() / np.abs(want).max() < 2e-5      # HIDDEN_TOL of fp32 models
 
 
+# CUDA-core path: an instance per number of rows; rows of one 256-element piece, of less and more than the pieces requested ahead.
+# A row's result does not depend on its companions, with SwiGLU in the gate/up kernel or in a launch of its own
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d_model,d_ffn", [(128, 136), (256, 264), (520, 768), (1032, 520)])
+def test_cuda_core_rows_do_not_depend_on_their_number(dtype, d_model, d_ffn):
+    shape = inputs.scaled(LAYER_F32, name="layer-rows", d_model=d_model, d_ffn=d_ffn, dtype=dtype)
+    w = inputs.make_weights(shape, 27, std=0.05)
+    page, max_seq, kvd = 16, 64, shape.n_kv_heads * shape.head_dim
+    k_hist, v_hist = inputs.make_kv(max_seq, kvd, 35, shape.dtype)
+    h = inputs.make_hidden(8, d_model, 60)
+    want = oracle_layer(shape, w, h, k_hist, v_hist, 21, max_seq)[0]
+    full = run_layer(shape, w, h, k_hist, v_hist, 21, max_seq, page, 0)
+    assert np.abs(full[0] - want).max() / np.abs(want).max() < HIDDEN_TOL[dtype]
+    for m in range(1, 8):
+        some = run_layer(shape, w, h[:m], k_hist, v_hist, 21, max_seq, page, 0)
+        assert all(np.array_equal(x, y[:m]) for x, y in zip(some, full)), m
+    assert binding.lib().sb_set_default_option(7, 2) == 0
+    try:
+        apart = run_layer(shape, w, h, k_hist, v_hist, 21, max_seq, page, 0)
+    finally:
+        binding.lib().sb_set_default_option(7, 3)
+    assert all(np.array_equal(x, y) for x, y in zip(full, apart))
+    # the exit test: the same rows alone and together
+    lm, gain = head_weights(inputs.scaled(shape, vocab=1000), 12)
+    every = run_exit(inputs.scaled(shape, vocab=1000), lm, gain, h, 1.5, 0)
+    for m in (1, 2, 3, 5, 6, 7):
+        some = run_exit(inputs.scaled(shape, vocab=1000), lm, gain, h[:m], 1.5, 0)
+        assert all(np.array_equal(x, y[:m]) for x, y in zip(some, every)), m
+
+
 @pytest.mark.parametrize("first_pos,m", [(40, 5), (1100, 3)])
 def test_layer_chain_equals_single_layer_calls(first_pos, m):
     """sb_k_layer_chain (n layers in one launch sequence, optionally with the rotation-angle table of sb_k_rope_table) gives
