@@ -12,6 +12,9 @@
 //                        tensor-memory buffer of its own and is added to the row's fp32 sums in registers (rounded, where
 //                        accumulating on in the tensor core over the whole context would truncate; and the rescaling by
 //                        the running maximum needs no pass over tensor memory).
+// The low halves' products go into a sum first: the tensor core truncates as it accumulates, and behind the high halves every
+// step of the low ones would be cut at the size of the whole sum.  Hidden state of a 7B layer after 100 prompt rows against
+// 64 bits: 9.2e-6 high halves first, 8.9e-6 low halves first (8.9e-6 in two sums of their own).
 //
 // Warp 0 brings the K and V blocks (TMA boxes of a page's rows, 128-byte swizzle, two stages each), warp 1 issues the
 // MMAs: S of the next block goes in front of P V of the current one, so the tensor pipe works while the softmax warps
@@ -145,12 +148,12 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
                     if (!(ok = mbar_wait(kfull(b), turn(blk), &abort_s, a.status, 7u))) break;
                     tc_fence_after();
 #pragma unroll
-                    for (int part = 0; part < 2; ++part)             // high halves, low halves
+                    for (int part = 1; part >= 0; --part)            // low halves, high halves (see the head of the file)
 #pragma unroll
                         for (int ks = 0; ks < HD / 16; ++ks) {
                             const uint32_t off = (uint32_t)((ks >> 2) * kPfHalf + (ks & 3) * 32);
                             tc_mma(s_col(b), smem_desc(q_s + part * kOp + off), smem_desc(k_s + b * kOp + off), idesc_n(kPfBlock),
-                                   (part > 0 || ks > 0) ? 1u : 0u);
+                                   (part < 1 || ks > 0) ? 1u : 0u);
                         }
                     tc_commit(kempty(b));
                     tc_commit(sfull(b));
@@ -161,12 +164,12 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
                     if (!(ok = mbar_wait(vfull(b), turn(pb), &abort_s, a.status, 7u))) break;
                     tc_fence_after();
 #pragma unroll
-                    for (int part = 0; part < 2; ++part)
+                    for (int part = 1; part >= 0; --part)
 #pragma unroll
                         for (int ks = 0; ks < kPfBlock / 16; ++ks)   // P: of 32 positions, 16 columns of high halves, then 16 of low halves
                             tc_mma_ts(o_col(b), s_col(b) + (uint32_t)((ks >> 1) * 32 + part * 16 + (ks & 1) * 8),
                                       smem_desc_mn(v_s + b * kOp + ks * 2048, kPfHalf), idesc_n(HD) | (1u << 16),
-                                      (part > 0 || ks > 0) ? 1u : 0u);
+                                      (part < 1 || ks > 0) ? 1u : 0u);
                     tc_commit(vempty(b));
                     tc_commit(ofull(b));
                 }
@@ -199,7 +202,9 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
         auto warp_wait = [&](uint32_t bar, uint32_t parity) {
             return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_s, a.status, 8u)) != 0;
         };
-        // probabilities as powers of two of (score - maximum) * scale * log2 e: one multiply-add and one exponential each
+        // probabilities as powers of two of (score - maximum) * scale * log2 e, the difference first: its rounding is the
+        // difference's own size, where scaled scores and maxima far from zero would each bring one of theirs, and the
+        // rescaling factor of the sums uses the same differences
         const float scale2 = attn_score_scale(HD) * 1.4426950408889634f;
         const int my_pos = a.pos0 + row0 + r;
         float m = -INFINITY, l = 0.f, f_prev = 0.f;
@@ -242,7 +247,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
                 }
             }
             const float nm = fmaxf(m, mx);
-            const float f = nm > -INFINITY ? exp2_flush((m - nm) * scale2) : 1.f, off = nm > -INFINITY ? nm * scale2 : 0.f;
+            const float f = nm > -INFINITY ? exp2_flush((m - nm) * scale2) : 1.f, top = nm > -INFINITY ? nm : 0.f;
             float ls[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
             for (int c = 0; c < kPfBlock; c += 32) {
@@ -251,7 +256,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
                 tc_wait_ld();
 #pragma unroll
                 for (int e = 0; e < 32; e += 2) {
-                    float p0 = exp2_flush(fmaf(__uint_as_float(v[e]), scale2, -off)), p1 = exp2_flush(fmaf(__uint_as_float(v[e + 1]), scale2, -off));
+                    float p0 = exp2_flush((__uint_as_float(v[e]) - top) * scale2), p1 = exp2_flush((__uint_as_float(v[e + 1]) - top) * scale2);
                     if (masked) {
                         p0 = c + e < seen ? p0 : 0.f;
                         p1 = c + e + 1 < seen ? p1 : 0.f;
