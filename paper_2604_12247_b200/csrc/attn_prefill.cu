@@ -38,6 +38,7 @@ constexpr int kPfBars = 15;
 
 struct alignas(64) PrefillAttnArgs {
     CUtensorMap tmK, tmV;      // the layer's page pool as [rows][Hkv * HD], boxes of box_rows x 64 channels
+    const __nv_bfloat16* v;    // the same pool as plain rows
     const float* q;            // [M][H * hd] rotated queries, row i at position pos0 + i
     const int* page_table;
     __nv_bfloat16* act_out;    // [block of 8 rows][16][H * hd]: high halves in rows 0-7, low halves in rows 8-15
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
     __shared__ uint32_t tmem_base_s;
     __shared__ volatile int abort_s;
     __shared__ __align__(8) unsigned long long bars_s[kPfBars];
+    __shared__ uint32_t not_finite_s[2][4];              // positions whose V row is not finite, in the (at most two) masked blocks
 
     const uint32_t raw = smem_u32(smem_raw), tiles = (raw + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
     uint8_t* const q_p = smem_raw + (tiles - raw);                             // [high | low] operand tiles of Q
@@ -92,6 +94,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
     const int n_blocks = last_pos / kPfBlock + 1;
     if (threadIdx.x == 0) {
         abort_s = 0;
+        for (int b = 0; b < 8; ++b) not_finite_s[b >> 2][b & 3] = 0u;
         for (int b = 0; b < 12; ++b) mbar_init(bars + 8u * b, 1);
         for (int b = 12; b < kPfBars; ++b) mbar_init(bars + 8u * b, 128);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -269,14 +272,45 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
             }
             l = l * f + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
             m = nm;
-            if (blk == n_blocks - 1 && last_pos + 1 < (blk + 1) * kPfBlock) {
-                // V rows beyond the last position: their probabilities are 0, and 0 * garbage must stay 0
+            if (masked) {
+                // V rows that some row of the tile does not see: its probability is 0, and 0 * V must stay 0.  Thread r looks
+                // at row r of the block: past the last position it may hold anything and becomes 0; of the others, channels
+                // that are not finite become 0 and the position is remembered for the rows that do see it.
                 if (!(ok = warp_wait(vfull(blk & 1), turn(blk)))) break;
-                if (blk * kPfBlock + r > last_pos) {
+                const int t = blk * kPfBlock + r;
+                auto piece_p = [&](int piece) {
+                    return reinterpret_cast<uint4*>(v_p + (blk & 1) * kOp + (piece >> 3) * kPfHalf + r * 128 + (((piece & 7) ^ (r & 7)) << 4));
+                };
+                bool finite = true;
+                if (t > last_pos) {
 #pragma unroll
-                    for (int piece = 0; piece < NH * 8; ++piece)
-                        *reinterpret_cast<uint4*>(v_p + (blk & 1) * kOp + (piece >> 3) * kPfHalf + r * 128 + (piece & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    for (int piece = 0; piece < NH * 8; ++piece) *piece_p(piece) = make_uint4(0u, 0u, 0u, 0u);
+                } else if (t > a.pos0 + row0) {
+                    const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+                    __nv_bfloat162 z = zero;             // 0 * v + z: stays 0 until a v is not finite
+#pragma unroll
+                    for (int piece = 0; piece < NH * 8; ++piece) {
+                        const uint4 w = *piece_p(piece);
+                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.x), zero, z);
+                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.y), zero, z);
+                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.z), zero, z);
+                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.w), zero, z);
+                    }
+                    finite = !(__hisnan(z.x) || __hisnan(z.y));
+                    if (!finite) {
+                        auto clean = [](uint32_t w) {
+                            return ((w & 0x7f80u) == 0x7f80u ? 0u : w & 0xffffu) | ((w & 0x7f800000u) == 0x7f800000u ? 0u : w & 0xffff0000u);
+                        };
+#pragma unroll 1
+                        for (int piece = 0; piece < NH * 8; ++piece) {
+                            uint4 w = *piece_p(piece);
+                            w.x = clean(w.x); w.y = clean(w.y); w.z = clean(w.z); w.w = clean(w.w);
+                            *piece_p(piece) = w;
+                        }
+                    }
                 }
+                const uint32_t found = __ballot_sync(0xffffffffu, !finite);
+                if (lane == 0) not_finite_s[n_blocks - 1 - blk][quad] = found;
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
             tc_wait_st();
@@ -286,6 +320,23 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
             f_prev = f;
         }
         if (ok) ok = take(n_blocks - 1, f_prev);
+        asm volatile("bar.sync 1, 128;" ::: "memory");   // not_finite_s of all four warps (reached by each of them, whatever it waited for)
+#pragma unroll 1
+        for (int b = 0; b < 8; ++b) {
+#pragma unroll 1
+            for (uint32_t left = not_finite_s[b >> 2][b & 3]; left; left &= left - 1) {
+                const int t = (n_blocks - 1 - (b >> 2)) * kPfBlock + (b & 3) * 32 + __ffs(left) - 1;
+                if (t > my_pos) continue;                // (a visible channel that is not finite decides the sum: its weight does not matter)
+                const uint32_t* row = reinterpret_cast<const uint32_t*>(
+                    a.v + ((size_t)a.page_table[t >> a.page_shift] * a.page + (t & (a.page - 1))) * (a.Hkv * HD) + kvh * HD);
+#pragma unroll
+                for (int e = 0; e < HD; e += 2) {
+                    const uint32_t w = __ldcg(row + (e >> 1));
+                    if ((w & 0x7f80u) == 0x7f80u) acc[e] += __uint_as_float(w << 16);
+                    if ((w & 0x7f800000u) == 0x7f800000u) acc[e + 1] += __uint_as_float(w & 0xffff0000u);
+                }
+            }
+        }
         if (ok && r < n_rows) {
             const int row = row0 + r, blk8 = row / kMaxW, i = row - blk8 * kMaxW;
             __nv_bfloat16* dst = a.act_out + ((size_t)blk8 * 16 + i) * qd + (size_t)h * HD;
@@ -333,6 +384,7 @@ bool launch_attention_prefill(cudaStream_t st, const float* q, const void* k_cac
                               unsigned int* status) {
     if (hd != 64 && hd != 128) return false;
     PrefillAttnArgs a;
+    a.v = static_cast<const __nv_bfloat16*>(v_cache);
     a.q = q; a.page_table = page_table; a.act_out = static_cast<__nv_bfloat16*>(act_out);
     a.H = H; a.Hkv = Hkv; a.page = page; a.page_shift = page_shift; a.pos0 = pos0; a.M = M; a.status = status;
     a.box_rows = page < kPfBlock ? page : kPfBlock;   // rows of one page, at most a block (pages are powers of two of 16 rows or more)

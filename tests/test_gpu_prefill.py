@@ -2,8 +2,11 @@
 oracle.  What prefill leaves behind is the K/V cache of every layer and the first generated token; both are checked
 through what is computed from them: the first token, the hidden state of that token after every layer (it attends
 over all cached prompt positions of each layer), and the tokens decoded afterwards."""
+import ctypes
+
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle
 from paper_2604_12247_b200 import binding, inputs
@@ -62,6 +65,41 @@ HD128_BF16 = inputs.scaled(SMALL_BF16, name="small-bf16-hd128", n_heads=4, n_kv_
 @pytest.mark.parametrize("n_prompt,kv_page", [(127, 16), (128, 128), (129, 256), (300, 32), (300, 64)])
 def test_tiled_attention_over_pages_and_head_widths(shape, n_prompt, kv_page):
     _wide_against_narrow_and_oracle(shape, n_prompt, 1, kv_page)
+
+
+def _kv_cache(ctx, max_seq, kv_page):
+    """K and V of all layers, [2, layers, positions, channels], out of the end of the context's workspace."""
+    s = ctx.shape
+    pages = -(-max_seq // kv_page)
+    count = s.n_layers * pages * kv_page * s.n_kv_heads * s.head_dim
+    assert 2 * count % 1024 == 0
+    base = -ctx.workspace.data_ptr() % 1024
+    end = base + binding.lib().sb_workspace_bytes(ctypes.byref(ctx.cfg))
+    kv = ctx.workspace[end - 4 * count:end].view(torch.bfloat16)
+    return kv.view(2, s.n_layers, pages * kv_page, -1).float().cpu()
+
+
+# a token whose hidden state is not a number (its embedding is infinite), inside the tiled attention's first and second
+# 128-row tile, at a block's first and last position, and last of the prompt: it reaches the positions from its own on, and
+# leaves those before it bit for bit as they are without it
+@pytest.mark.parametrize("shape", [SMALL_BF16, HD128_BF16], ids=lambda s: s.name)
+@pytest.mark.parametrize("n_prompt,at", [(200, 70), (200, 127), (200, 128), (200, 150), (200, 199), (520, 300), (100, 40)])
+def test_a_token_that_is_not_finite_stays_out_of_earlier_positions(shape, n_prompt, at):
+    w = inputs.make_weights(shape, 5, damp_rho=0.3)
+    w["embed"][7] = float("inf")
+    pr = inputs.make_prompt(shape, n_prompt, 17).numpy()
+    pr[pr == 7] = 8
+    ctx, _ = gpu_ctx(shape, w, 544, gemm=1)
+    ctx.prefill(pr)
+    clean = _kv_cache(ctx, 544, 16)
+    ctx.reset()
+    pr[at] = 7
+    ctx.prefill(pr)
+    got = _kv_cache(ctx, 544, 16)
+    assert torch.equal(got[:, :, :at], clean[:, :, :at])
+    assert not torch.isfinite(got[:, 0, at]).any() and torch.isfinite(got[:, 0, at + 1:n_prompt]).all()
+    assert not torch.isfinite(got[:, 1:, at:n_prompt]).any()
+    ctx.close()
 
 
 def _wide_against_narrow_and_oracle(shape, n_prompt, wide_mode, kv_page=16):
