@@ -201,8 +201,8 @@ static size_t carve(const Dims& D, char* base, bool with_state, Work* w) {
             W.pf_attn_stride = (size_t)max_chunks * kMaxW * D.H * (D.hd + 2);
             const int tiles = (int)rows / kTileRowsPf;
             size_t floats = (size_t)kWideBlocks * W.pf_attn_stride;
-            for (size_t n : {tc_wide_partial_rows(D.d, tiles) * (D.qd + 2 * D.kvd), tc_wide_partial_rows(D.qd, tiles) * D.d,
-                             tc_wide_partial_rows(D.F, tiles) * D.d})
+            for (size_t n : {tc_wide_partial_floats(D.d, (size_t)D.qd + 2 * D.kvd, tiles), tc_wide_partial_floats(D.qd, (size_t)D.d, tiles),
+                             tc_wide_partial_floats(D.F, (size_t)D.d, tiles)})
                 if (n > floats) floats = n;
             c.take(W.pf_part, sizeof(float) * floats);
         }

@@ -857,33 +857,41 @@ static int choose_pair_half(int n_rows, int G) {
 static int g_pair_floor_rows = 96, g_pair_split_pm = 30;
 static int pair_floor_rows(int n_tiles) { return n_tiles > 1 ? kTileRows : g_pair_floor_rows; }
 // Passes of several tiles: k blocks that one accumulator takes in at most (where the matrix is split at all).  The tensor
-// core truncates as it accumulates, so the error of a sum grows with its length: the balance would be as good unsplit, but
-// 64 and 86 k blocks per sum moved the hidden state after a 512-token prompt (7B shape, 6 seeds) to 1.02e-4 from its fp64
-// value, against 0.68e-4 with sums of 16 to 43.
-constexpr int kWideMaxChain = 45;
+// core truncates as it accumulates, so the error of a sum grows with its length, though the balance would be as good with fewer
+// splits.  Hidden state from its fp64 value, 7B shape, after 512 / 300 prompt rows (6 / 4 seeds): QKV, output and down
+// projections unsplit (64, 64, 172 k blocks) 1.0e-4 / -, in sums of 32, 32, 43 7.2e-5 / 8.0e-5, of 22, 22, 43 6.8e-5 / 6.4e-5, as in
+// passes of one tile (6.8e-5 / 6.4e-5), whose matrices of up to 66 k blocks have sums of 22; shorter ones gain no more (4 splits
+// 6.4e-5 / 6.8e-5).  13B shape, sums of 40, 16, 36 1.4e-4, in passes of one tile (80, 27, 72) 2.1e-4.
+constexpr int kWideMaxChain = 45, kWideShortK = 66, kWideShortChain = 22;
 static int wide_min_splits(int KB) {
-    const int s = (KB + kWideMaxChain - 1) / kWideMaxChain;
+    const int chain = KB <= kWideShortK ? kWideShortChain : kWideMaxChain, s = (KB + chain - 1) / chain;
     return s < kMaxSplit ? s : kMaxSplit;   // consumers sum at most kMaxSplit partials
 }
-// Most k splits of a wide GEMM: 8 for one tile; with more, what 8 splits of one tile or the fewest allowed splits of all of
-// them write (33 MB of partials for 512 rows of the 7B output projection: beside the weights they stay in L2).  A function
-// of k and the number of tiles only: the order of a prompt's sums must not depend on how long its context may grow.
-static int wide_max_splits(int KB, int n_tiles) {
+// Most k splits of a wide GEMM with n output columns: 8 for one tile; with more, as many as leave 60 MB of partials (which
+// stay in L2 for their consumer), or the fewest allowed.  A function of the matrix and the number of tiles only: the order of a
+// prompt's sums must not depend on how long its context may grow.
+constexpr size_t kWidePartialBytes = size_t(60) << 20;
+static int wide_max_splits(int KB, size_t n, int n_tiles) {
+    if (n_tiles == 1) return kMaxSplit;
+    const size_t fit = kWidePartialBytes / (sizeof(float) * kWideBlocks * kMaxW * n_tiles * n);
     const int least = wide_min_splits(KB);
-    return n_tiles * least > kMaxSplit ? least : kMaxSplit / n_tiles;
+    return fit >= (size_t)kMaxSplit ? kMaxSplit : (int)fit > least ? (int)fit : least;
 }
-size_t tc_wide_partial_rows(int K, int n_tiles) {
+size_t tc_wide_partial_floats(int K, size_t n, int n_tiles) {
     size_t most = 0;
     for (int t = 1; t <= n_tiles; ++t) {
-        const size_t rows = (size_t)t * kWideBlocks * kMaxW * wide_max_splits((K + kBK - 1) / kBK, t);
-        if (rows > most) most = rows;
+        const size_t floats = (size_t)t * kWideBlocks * kMaxW * n * wide_max_splits((K + kBK - 1) / kBK, n, t);
+        if (floats > most) most = floats;
     }
     return most;
 }
 static void choose_split_cta_pair(const int* n_rows, int n_mats, int KB, int G, int* R_out, int* S_out, int n_tiles = 1) {
     double best = 1e300;
     int bR = 128, bS = 1;
-    for (int S = n_tiles > 1 ? wide_min_splits(KB) : 1; S <= wide_max_splits(KB, n_tiles) && S <= KB; ++S)
+    size_t n = 0;
+    for (int j = 0; j < n_mats; ++j) n += n_rows[j];
+    const int most = wide_max_splits(KB, n, n_tiles);
+    for (int S = n_tiles > 1 ? wide_min_splits(KB) : 1; S <= most && S <= KB; ++S)
         for (int R = 128; R >= 8; R -= 8) {
             long long chunks = 0;
             for (int j = 0; j < n_mats; ++j) chunks += (n_rows[j] + 2 * R - 1) / (2 * R);

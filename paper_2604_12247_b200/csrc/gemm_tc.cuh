@@ -31,8 +31,8 @@ bool tc_set_split_penalty(int per_mille);
 // wide passes (GemmArgs::nb > 1): true (default) = clusters of two CTAs sharing one activation tile (cta_group::2),
 // false = one CTA per work item
 void tc_set_wide_cta_pairs(bool on);
-// rows of fp32 partials (as wide as the output) that a wide GEMM over k = K of up to n_tiles 128-row tiles leaves at most
-size_t tc_wide_partial_rows(int K, int n_tiles);
+// floats of partials that a wide GEMM over k = K with n output columns leaves at most, for up to n_tiles 128-row tiles
+size_t tc_wide_partial_floats(int K, size_t n, int n_tiles);
 int tc_wide_rows();   // most prompt rows one wide pass can take under that setting on the current device
 // the work decomposition for `units` CTAs (modes 0, 1: 8-row kernel, its gate/up form) or clusters (modes 2, 3: CTA-pair
 // kernel on one tile, its gate/up form in items of one accumulator; + 256 * t: as the launches of a pass of t tiles have it):

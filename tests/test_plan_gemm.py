@@ -67,9 +67,9 @@ def test_wide_pass_plans(shape, tiles, units):
         assert R % 8 == 0 and 8 <= R <= 128 and 1 <= S <= min(8, kb), (name, R, S)
         assert items == sum(math.ceil(n / (2 * R)) for n in n_rows) * S * tiles
         if tiles > 1:
-            assert math.ceil(kb / S) <= 45, (name, S)                  # k blocks that one accumulator takes in
-            least = math.ceil(kb / 45)
-            assert S * tiles <= max(8, least * tiles), (name, S)       # rows of partials the workspace holds
+            assert math.ceil(kb / S) <= (45 if kb > 66 else 22), (name, S)     # k blocks that one accumulator takes in
+            least = math.ceil(kb / (45 if kb > 66 else 22))
+            assert S <= max(60 * 2**20 // (4 * 128 * tiles * sum(n_rows)), least), (name, S)     # partials the workspace has room for
         else:
             assert (R, S, items) == binding.plan_gemm(2, n_rows, k, units)
         busiest = math.ceil(items / units) * 2 * R * math.ceil(kb / S)
