@@ -33,8 +33,8 @@ def _hidden_after_prefill(ctx, prompt, n_layers):
     return first, hid
 
 
-# 16: the smallest wide pass; 64, 70, 100: one ragged wide pass (70 and 100 end in a partial block of 8 rows); 128: a
-# whole pass; 130: a whole pass + 2 rows through an 8-row pass; 300: two whole passes and a ragged one.  Page size 16
+# 16: two blocks of 8 rows; 64, 70, 100: one ragged tile (70 and 100 end in a partial block of 8 rows); 128: a whole tile;
+# 130: two tiles, 2 rows in the second; 300: three tiles.  (Modes 2 and 3 send a tile per pass.)  Page size 16
 # wide_mode 1: wide GEMMs on CTA pairs + the tiled tensor-core attention kernel (the default); 2: the decode attention
 # kernels; 3: as 1 with the wide GEMMs on single CTAs
 @pytest.mark.parametrize("wide_mode", [1, 2, 3])
@@ -65,6 +65,15 @@ HD128_BF16 = inputs.scaled(SMALL_BF16, name="small-bf16-hd128", n_heads=4, n_kv_
 @pytest.mark.parametrize("n_prompt,kv_page", [(127, 16), (128, 128), (129, 256), (300, 32), (300, 64)])
 def test_tiled_attention_over_pages_and_head_widths(shape, n_prompt, kv_page):
     _wide_against_narrow_and_oracle(shape, n_prompt, 1, kv_page)
+
+
+# FFN widths whose gate/up GEMM takes one tile of rows in one round of items in two parts (more than 128 columns per cluster):
+# just above that line, the 7B width and 8 columns more (a last item past the end), the Llama-3 width, and one that needs the
+# widest items there are; as many k blocks in the down projection as make it split in several (300 rows: three tiles)
+@pytest.mark.parametrize("d_ffn", [9480, 11008, 11016, 14336, 18816])
+@pytest.mark.parametrize("n_prompt", [33, 75, 128, 300])
+def test_wide_prefill_with_wide_ffn(d_ffn, n_prompt):
+    _wide_against_narrow_and_oracle(inputs.scaled(SMALL_BF16, name=f"wide-ffn-{d_ffn}", n_layers=3, d_ffn=d_ffn), n_prompt, 1)
 
 
 def _kv_cache(ctx, max_seq, kv_page):
@@ -148,7 +157,7 @@ def _wide_against_narrow_and_oracle(shape, n_prompt, wide_mode, kv_page=16):
 
 
 def test_wide_prefill_at_the_bench_shape_matches_narrow_first_token_and_tokens():
-    """7B shape, 200-token prompt (a whole wide pass + a ragged one of 72 rows): same first token and decoded tokens as the
+    """7B shape, 200-token prompt (one pass of two tiles, the second ragged): same first token and decoded tokens as the
     8-row passes (which the 7B-shape run tests compare with the oracle), in well under their time.  The wide passes
     themselves are compared with the oracle on the small model above and, at the 7B attention geometry with a 512-token
     prompt, by test_bench_lengths_on_7b_attention_geometry_match_oracle."""
