@@ -303,7 +303,7 @@ __device__ __forceinline__ void soft_final_merge(const SoftTriple* part, int n_c
         if (lane == 0) {
             float c = 1.f / t.s;   // the arg-max term contributes exp(0) = 1, so max softmax = 1 / sum
             conf[i] = c;
-            token[i] = t.idx;
+            token[i] = t.idx == soft_empty().idx ? 0 : t.idx;   // no logit is a number: a token the embedding can take all the same
             exit_flag[i] = c >= threshold ? 1 : 0;
         }
     }

@@ -2,12 +2,16 @@
 KV-page boundaries inside a round, widest rounds, full acceptance through the primitives."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle
 from paper_2604_12247_b200 import binding, inputs
 from gpu_util import gemm_modes, gpu_ctx
 
 pytestmark = pytest.mark.gpu
+
+BF16 = inputs.scaled(inputs.LLAMA3_8B, name="edges-bf16", n_layers=2, d_model=512, n_heads=8, n_kv_heads=2, head_dim=64,
+                     d_ffn=1408, vocab=2048)
 
 SMALL_BF16 = inputs.scaled(inputs.LLAMA3_8B, name="small-bf16", n_layers=4, d_model=512, n_heads=8, n_kv_heads=2,
                            head_dim=64, d_ffn=1408, vocab=2048, head_scale=16.0)
@@ -116,4 +120,19 @@ def test_bounded_device_wait_runs_out_and_context_survives(tiny_damped_weights):
     assert e.value.status == -5
     ctx.reset()
     assert np.array_equal(ctx.generate_ar(pr, 6)["tokens"], ref)
+    ctx.close()
+
+
+@pytest.mark.parametrize("shape", [inputs.RUNS["tiny-damped"].shape, BF16], ids=["f32", "bf16"])
+def test_logits_that_are_no_numbers_give_a_token_of_the_vocabulary(shape):
+    """Every place that embeds a token straight from device memory takes what the heads and the sampler leave there: with no
+    logit a number that is token 0, never an index outside the embedding."""
+    w = inputs.make_weights(shape, 3)
+    w["final_norm"] = torch.full_like(w["final_norm"], float("nan"))
+    ctx, _ = gpu_ctx(shape, w, 64)
+    pr = inputs.make_prompt(shape, 12, 3).numpy()
+    for sampling in ((0.0, 1.0), (1.0, 1.0), (1.0, 0.9)):
+        ctx.set_sampling(sampling[0], 5, sampling[1])
+        assert not ctx.generate_ar(pr, 6)["tokens"].any()
+        assert not ctx.generate(pr, 6, 1, 3, (1.0,), 0.3)["tokens"].any()
     ctx.close()
