@@ -35,6 +35,7 @@ constexpr int kPfBlock = 128;        // cached positions per block
 constexpr int kPfThreads = 6 * 32;   // producer, MMA issuer, four softmax warps
 constexpr int kPfHalf = 128 * 128;   // bytes of a 128-row x 64-channel operand tile (128-byte swizzle)
 constexpr int kPfBars = 15;
+constexpr size_t kPfOneCta = 116 * 1024;   // dynamic shared memory that two CTAs of an SM cannot both have (228 KB)
 
 struct alignas(64) PrefillAttnArgs {
     CUtensorMap tmK, tmV;      // the layer's page pool as [rows][Hkv * HD], boxes of box_rows x 64 channels
@@ -367,7 +368,9 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
 }
 
 template <int HD> static bool launch_hd(cudaStream_t st, const PrefillAttnArgs& a) {
-    const size_t smem = (size_t)6 * (HD / 64) * kPfHalf + 1024;
+    // More than half of an SM's shared memory, also where half would do (64 channels): a CTA takes all of the SM's tensor memory,
+    // and a second one on the SM would sit in its allocation, a wait without a limit, and hold back the next launch.
+    const size_t tiles = (size_t)6 * (HD / 64) * kPfHalf + 1024, smem = tiles > kPfOneCta ? tiles : kPfOneCta;
     static bool configured[kMaxDevices];             // function attributes are per device
     const int dev = current_device();
     if (dev < 0) return false;
