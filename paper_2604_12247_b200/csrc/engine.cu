@@ -2,6 +2,7 @@
 // of Section 3.3 and the C ABI declared in include/specbound.h.  Every arithmetic step runs in a
 // kernel; the host only sequences launches and reads the few integers that gate the next launch
 // (exit flag after a probe, acceptance count after a round).
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -31,6 +32,25 @@ static TcPlanCache& stateless_plans() {
     TcPlanCache& c = cache[dev < 0 ? 0 : dev];
     if (c.plans.size() > 512) c.clear();
     return c;
+}
+
+// The kernels already asked for, per device: one open-addressed table for the whole library (it has about 200 kernels), filled
+// without a lock, since contexts may be launched from several threads.  A full table asks again at every launch.
+void ask_max_carveout(const void* kernel) {
+    constexpr size_t kSlots = 512;
+    static std::atomic<const void*> asked[kMaxDevices][kSlots];
+    const int dev = current_device();
+    if (dev < 0) return;
+    const size_t at = ((uintptr_t)kernel >> 4) % kSlots;
+    for (size_t i = 0; i < kSlots; ++i) {
+        std::atomic<const void*>& slot = asked[dev][(at + i) % kSlots];
+        const void* held = slot.load(std::memory_order_acquire);
+        if (held == kernel) return;
+        if (held) continue;
+        cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (slot.compare_exchange_strong(held, kernel) || held == kernel) return;
+    }
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
 }
 
 struct Tracer {

@@ -144,6 +144,8 @@ inline int device_sm_count() {   // SMs of the current device (148 if the query 
     if (!n[dev] && (cudaDeviceGetAttribute(&n[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n[dev] <= 0)) n[dev] = 148;
     return n[dev];
 }
+// Asks for the maximal shared-memory carve-out of a kernel, once per kernel and device (engine.cu).
+void ask_max_carveout(const void* kernel);
 // cluster with more than one CTA: launches thread-block clusters of that shape (the grid must be a multiple of it);
 // pdl: launch with programmatic stream serialisation (the kernel may start while its predecessor drains)
 template <typename... KArgs, typename... Args>
@@ -168,18 +170,8 @@ inline cudaError_t launch_kcp(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.attrs = attr;
     cfg.numAttrs = n_attr;
     // every kernel asks for the same (maximal) shared-memory carve-out: an SM never has to drain to
-    // change its L1/shared split between two kernels of the chain.  Function attributes are per device.
-    static void* seen[kMaxDevices][32];
-    static int n_seen[kMaxDevices];
-    const int dev = current_device();
-    if (dev >= 0) {
-        bool known = false;
-        for (int i = 0; i < n_seen[dev]; ++i) known |= seen[dev][i] == (void*)kernel;
-        if (!known) {
-            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-            if (n_seen[dev] < 32) seen[dev][n_seen[dev]++] = (void*)kernel;
-        }
-    }
+    // change its L1/shared split between two kernels of the chain.
+    ask_max_carveout((const void*)kernel);
     return report_cuda("kernel launch", cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
 }
 // clusters of cluster_y CTAs along y
