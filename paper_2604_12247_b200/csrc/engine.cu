@@ -210,7 +210,7 @@ static size_t carve(const Dims& D, char* base, bool with_state, Work* w) {
     if (with_state) {
         c.take(W.toks, sizeof(int) * (D.max_seq + 16));
         c.take(W.logits, sizeof(float) * (size_t)kMaxW * D.V);
-        c.take(W.sample_e, sizeof(double) * (size_t)kMaxW * D.V);
+        c.take(W.sample_e, sample_scratch_bytes(kMaxW, D.V));
         if (!D.f32) {
             const size_t rows = (size_t)wide_rows(D.max_seq);
             c.take(W.pf_h, sizeof(float) * rows * D.d);
@@ -1195,7 +1195,7 @@ int sb_k_exit_confidence(const sb_config* cfg, const void* h, int32_t m, const v
 // Sampling kernel alone: tokens of m rows of device logits.  Nothing is published to the host, so the kernel's
 // completion counter is not used: the call touches the caller's buffers only.
 size_t sb_k_sample_scratch_bytes(int32_t m, int32_t vocab) {
-    return m < 1 || vocab < 1 ? 0 : 2 * sizeof(double) * (size_t)m * (size_t)vocab;   // the exponentials take half of it
+    return m < 1 || vocab < 1 ? 0 : sample_scratch_bytes(m, vocab);
 }
 
 int sb_k_sample(const float* logits, int32_t m, int32_t vocab, float temperature, float top_p, uint64_t seed, int64_t pos0,

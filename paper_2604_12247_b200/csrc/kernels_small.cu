@@ -923,7 +923,6 @@ __device__ __forceinline__ unsigned int peer_ld_u32(uint32_t addr) {
 }
 
 constexpr int kSampleListMax = 512;          // tokens of one bucket that the first CTA compares with one another
-constexpr int kSampleSmemVocab = 131072;     // largest vocabulary whose exponentials (an eighth per CTA) stay in shared memory
 
 // What the select of the nucleus threshold keeps in shared memory.
 struct SelectShared {

@@ -332,6 +332,11 @@ __host__ __device__ inline double sample_uniform(unsigned long long seed, long l
     return ((double)(sample_hash(seed, pos) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
 }
 constexpr int kSampleMaxVocab = 262144;
+constexpr int kSampleSmemVocab = 131072;     // largest vocabulary whose exponentials (an eighth per CTA) stay in shared memory
+// device memory for the exponentials of m rows (never nothing: callers hand over a pointer)
+inline size_t sample_scratch_bytes(int m, int vocab) {
+    return sizeof(double) * (vocab > kSampleSmemVocab ? (size_t)m * (size_t)vocab : 1);
+}
 struct SampleArgs {
     const float* logits;       // [m][V] final logits, row r0 first
     double* e;                 // [m][V] scratch: exp((z - row max) / temperature), where it does not fit shared memory
