@@ -231,11 +231,54 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
         };
         bool ok = true;
         for (int blk = 0; blk < n_blocks; ++blk) {
+            const bool masked = blk * kPfBlock + kPfBlock - 1 > a.pos0 + row0;
+            if (masked) {
+                // V rows that some row of the tile does not see: its probability is 0, and 0 * V must stay 0.  Thread r looks
+                // at row r of the block: past the last position it may hold anything and becomes 0; of the others, channels
+                // that are not finite become 0 and the position is remembered for the rows that do see it.  (In front of the
+                // wait for the block's scores: the tensor core is at them.)
+                if (!(ok = warp_wait(vfull(blk & 1), turn(blk)))) break;
+                const int t = blk * kPfBlock + r;
+                auto piece_p = [&](int piece) {
+                    return reinterpret_cast<uint4*>(v_p + (blk & 1) * kOp + (piece >> 3) * kPfHalf + r * 128 + (((piece & 7) ^ (r & 7)) << 4));
+                };
+                bool finite = true;
+                if (t > last_pos) {
+#pragma unroll
+                    for (int piece = 0; piece < NH * 8; ++piece) *piece_p(piece) = make_uint4(0u, 0u, 0u, 0u);
+                } else if (t > a.pos0 + row0) {
+                    const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+                    __nv_bfloat162 z[4] = {zero, zero, zero, zero};   // 0 * v + z: stays 0 until a v is not finite
+#pragma unroll
+                    for (int piece = 0; piece < NH * 8; ++piece) {
+                        const uint4 w = *piece_p(piece);
+                        z[0] = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.x), zero, z[0]);
+                        z[1] = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.y), zero, z[1]);
+                        z[2] = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.z), zero, z[2]);
+                        z[3] = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.w), zero, z[3]);
+                    }
+                    z[0] = __hadd2(__hadd2(z[0], z[1]), __hadd2(z[2], z[3]));
+                    finite = !(__hisnan(z[0].x) || __hisnan(z[0].y));
+                    if (!finite) {
+                        auto clean = [](uint32_t w) {
+                            return ((w & 0x7f80u) == 0x7f80u ? 0u : w & 0xffffu) | ((w & 0x7f800000u) == 0x7f800000u ? 0u : w & 0xffff0000u);
+                        };
+#pragma unroll 1
+                        for (int piece = 0; piece < NH * 8; ++piece) {
+                            uint4 w = *piece_p(piece);
+                            w.x = clean(w.x); w.y = clean(w.y); w.z = clean(w.z); w.w = clean(w.w);
+                            *piece_p(piece) = w;
+                        }
+                    }
+                }
+                const uint32_t found = __ballot_sync(0xffffffffu, !finite);
+                if (lane == 0) not_finite_s[n_blocks - 1 - blk][quad] = found;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
             if (!(ok = warp_wait(sfull(blk & 1), turn(blk)))) break;
             tc_fence_after();
             const uint32_t s0 = s_col(blk & 1) + lanes;
             const int seen = my_pos - blk * kPfBlock + 1;   // visible positions of the block (maybe more than it has, or none)
-            const bool masked = blk * kPfBlock + kPfBlock - 1 > a.pos0 + row0;
             float mx = -INFINITY;
 #pragma unroll 1
             for (int c = 0; c < kPfBlock; c += 32) {
@@ -273,47 +316,6 @@ __global__ void __launch_bounds__(kPfThreads, 1) k_attn_prefill(const __grid_con
             }
             l = l * f + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
             m = nm;
-            if (masked) {
-                // V rows that some row of the tile does not see: its probability is 0, and 0 * V must stay 0.  Thread r looks
-                // at row r of the block: past the last position it may hold anything and becomes 0; of the others, channels
-                // that are not finite become 0 and the position is remembered for the rows that do see it.
-                if (!(ok = warp_wait(vfull(blk & 1), turn(blk)))) break;
-                const int t = blk * kPfBlock + r;
-                auto piece_p = [&](int piece) {
-                    return reinterpret_cast<uint4*>(v_p + (blk & 1) * kOp + (piece >> 3) * kPfHalf + r * 128 + (((piece & 7) ^ (r & 7)) << 4));
-                };
-                bool finite = true;
-                if (t > last_pos) {
-#pragma unroll
-                    for (int piece = 0; piece < NH * 8; ++piece) *piece_p(piece) = make_uint4(0u, 0u, 0u, 0u);
-                } else if (t > a.pos0 + row0) {
-                    const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
-                    __nv_bfloat162 z = zero;             // 0 * v + z: stays 0 until a v is not finite
-#pragma unroll
-                    for (int piece = 0; piece < NH * 8; ++piece) {
-                        const uint4 w = *piece_p(piece);
-                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.x), zero, z);
-                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.y), zero, z);
-                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.z), zero, z);
-                        z = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&w.w), zero, z);
-                    }
-                    finite = !(__hisnan(z.x) || __hisnan(z.y));
-                    if (!finite) {
-                        auto clean = [](uint32_t w) {
-                            return ((w & 0x7f80u) == 0x7f80u ? 0u : w & 0xffffu) | ((w & 0x7f800000u) == 0x7f800000u ? 0u : w & 0xffff0000u);
-                        };
-#pragma unroll 1
-                        for (int piece = 0; piece < NH * 8; ++piece) {
-                            uint4 w = *piece_p(piece);
-                            w.x = clean(w.x); w.y = clean(w.y); w.z = clean(w.z); w.w = clean(w.w);
-                            *piece_p(piece) = w;
-                        }
-                    }
-                }
-                const uint32_t found = __ballot_sync(0xffffffffu, !finite);
-                if (lane == 0) not_finite_s[n_blocks - 1 - blk][quad] = found;
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            }
             tc_wait_st();
             tc_fence_before();                           // (and behind the loads of P V in the previous step)
             mbar_arrive(pready(blk & 1));
