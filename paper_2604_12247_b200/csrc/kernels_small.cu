@@ -865,532 +865,6 @@ void launch_accept(cudaStream_t st, const int* g, const int* drafts8, int w, int
     launch_k(k_accept, dim3(1), dim3(64), 0, st, g, d, w, max_emit, result, mirror);
 }
 
-// ------------------------------------------------------------------------------------------------
-// Sampling decoding (Section 4.3, decoding strategies): token = inverse CDF, in vocabulary order, of
-// softmax(z / temperature), restricted to its top-p nucleus when top_p < 1, at the uniform number of the
-// token's sequence position.  One cluster of 8 CTAs per row; every CTA owns a slice of whole 128-token cells.
-//
-//  1. A thread keeps its tokens' logits in registers (a warp owns whole cells).  Slice maxima are exchanged through
-//     distributed shared memory; e_v = exp((z_v - max) / T) in fp64 stays in the CTA's shared memory (in a scratch row in
-//     L2 for the vocabularies whose slice does not fit), where everything below reads it, the last step included.
-//  2. Nucleus (top_p < 1): {v : z_v >= z*}, z* the largest logit whose upper set holds top_p of the mass (equal
-//     logits enter together), masses as 2^40 fixed-point integers (exact and order-free).  One histogram of the mass over
-//     2048 buckets linear in the logit, from the maximum down to the lightest token that can decide anything (tokens
-//     lighter than (1 - top_p) * total / V cannot and skip it): any monotone bucket rule selects the same z*, and this one
-//     spreads the tokens, where buckets by the logits' leading bits put a quarter of them on one word and waited for the
-//     shared-memory atomics.  Every CTA sums its share of the buckets over the 8 histograms out of its peers' shared
-//     memory and hands the sums to every CTA; every CTA scans the buckets from the top and finds the same one.  The last bucket
-//     ends at the minimum where that comes first, so that nearly flat rows are spread too.  The few
-//     tokens of that bucket go to the first CTA, which finds z* among them by comparing all pairs.  Where they are too
-//     many for that (many tied logits, or a flat part far below the maximum), z* is their one key, or is found by a radix
-//     select over their range of order-preserving 32-bit keys, 11 bits at a time from the top, on the same histograms.
-//  3. CDF walk: every CTA sums its cells' nucleus members (a warp per cell, fixed shuffle tree, fp64) and hands the sums
-//     to every CTA; every CTA scans the cell sums in order, exactly one thread owns the interval holding u * total
-//     (neighbouring intervals are built from the same additions), and the CTA that owns that cell walks it with one warp.
-//
-// fp64 sums and exponentials: for equal logits the token can differ from an fp64 reference only by summation
-// order.  Everything is a pure function of (logits, u): deterministic.  All waits are hardware barriers.
-// Bound: latency (6 rows of 128256 logits are half a microsecond of HBM time): what counts are the cluster barriers, the
-// fp64 exponentials and the shared-memory atomics.  6 rows, top_p 0.9, us as a radix select over the key bits for every row
-// (exponentials and masses in L2) / now: V = 32000 24.7 / 14.7, 128256 43.2 / 27.6, 262144 67 / 47; nearly flat rows (standard
-// deviation 0.01) 25.2 / 15.3, 45 / 29.5, 70 / 52; one token far above nearly flat ones 25 / 26, 45 / 46, 70 / 78; top_p 1:
-// 128256 17.1 / 14.5.
-// ------------------------------------------------------------------------------------------------
-constexpr int kSampleThreads = 1024;
-constexpr int kSampleCell = 128;
-constexpr int kSampleMaxCells = kSampleMaxVocab / kSampleCell;
-constexpr int kSampleCtas = 8;
-constexpr int kSelectBuckets = 2048;
-
-__device__ __forceinline__ unsigned long long hist_mass(unsigned int h0, unsigned int h1, unsigned int h2) {
-    return (unsigned long long)h0 + ((unsigned long long)h1 << 14) + ((unsigned long long)h2 << 28);
-}
-// larger logit <-> larger key; -0 and +0 share a key
-__device__ __forceinline__ unsigned int order_key(float z) {
-    const unsigned int b = __float_as_uint(z + 0.0f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-// address of `local` (a shared-memory object of this kernel) in the CTA of cluster rank `rank`
-__device__ __forceinline__ uint32_t peer_smem(const void* local, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(local)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ unsigned int peer_ld_u32(uint32_t addr) {
-    unsigned int v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-
-constexpr int kSampleListMax = 512;          // tokens of one bucket that the first CTA compares with one another
-
-// What the select of the nucleus threshold keeps in shared memory.
-struct SelectShared {
-    // mass histogram in three 14-bit parts (a part's bucket sum stays below 2^32 for up to 262144 tokens):
-    // mass of bucket b = hist[0][b] + (hist[1][b] << 14) + (hist[2][b] << 28)
-    unsigned int hist[3][kSelectBuckets];
-    union {
-        unsigned long long merged[kSelectBuckets];  // the row's bucket masses
-        double cell[kSampleMaxCells];               // afterwards: every cell's sum
-    };
-    unsigned long long wsum[32], above;
-    unsigned long long target, light;               // mass wanted; mass of the lightest token that can decide anything
-    float mx, per_unit;                             // the rule of the first histogram's buckets
-    unsigned int digit, lo, hi;
-};
-__device__ __forceinline__ unsigned long long sample_mass(double e) { return __double2ull_rn(e * 1099511627776.0); }   // 2^40 fixed point: integer sums are exact in any order
-// adds the mass q of this thread's token to bucket b (-1: none); all lanes of the warp together
-__device__ __forceinline__ void select_add(SelectShared& s, int b, unsigned long long q) {
-    unsigned int p0 = b < 0 ? 0u : (unsigned int)(q & 0x3fffull), p1 = b < 0 ? 0u : (unsigned int)((q >> 14) & 0x3fffull),
-                 p2 = b < 0 ? 0u : (unsigned int)(q >> 28);
-    // equal buckets across the whole warp (flat or heavily tied logits) would serialise 32 atomics on
-    // one word: merge them first (exact integer reductions); otherwise one atomic per lane and part
-    const bool uniform = __all_sync(0xffffffffu, b == __shfl_sync(0xffffffffu, b, 0));
-    if (uniform) {
-        p0 = __reduce_add_sync(0xffffffffu, p0);
-        p1 = __reduce_add_sync(0xffffffffu, p1);
-        p2 = __reduce_add_sync(0xffffffffu, p2);
-    }
-    if (b >= 0 && (!uniform || (threadIdx.x & 31) == 0)) {
-        if (p0) atomicAdd(&s.hist[0][b], p0);
-        if (p1) atomicAdd(&s.hist[1][b], p1);
-        if (p2) atomicAdd(&s.hist[2][b], p2);
-    }
-}
-// Bucket masses of the whole row: this CTA sums its share of the buckets (an eighth) over the 8 histograms and hands each
-// sum to every CTA's table; integer sums, the same numbers everywhere.
-__device__ __forceinline__ void select_merge(SelectShared& s, int rank) {
-    cluster_sync_all();                             // every CTA's histogram is complete
-    constexpr int share = kSelectBuckets / kSampleCtas;
-    if (threadIdx.x < share) {
-        const int b = rank * share + (int)threadIdx.x;
-        unsigned int hh[kSampleCtas][3];
-#pragma unroll
-        for (int r = 0; r < kSampleCtas; ++r) {
-            const uint32_t base = peer_smem(&s.hist[0][0], r);
-#pragma unroll
-            for (int part = 0; part < 3; ++part) hh[r][part] = peer_ld_u32(base + 4u * (uint32_t)(part * kSelectBuckets + b));
-        }
-        unsigned long long mass = 0ull;
-#pragma unroll
-        for (int r = 0; r < kSampleCtas; ++r) mass += hist_mass(hh[r][0], hh[r][1], hh[r][2]);
-#pragma unroll
-        for (int r = 0; r < kSampleCtas; ++r)
-            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_smem(&s.merged[b], r)), "l"(mass) : "memory");
-    }
-    cluster_sync_all();                             // every CTA's table of merged bucket masses is complete
-}
-// Walks the buckets from the top (bucket_at(p) = the p-th from the top): a CTA-wide scan, thread t owns positions 2t and 2t+1.
-// Leaves the bucket in which the mass reaches the target in digit, the mass above it in above, and calls found(bucket, its
-// mass) in one thread; every CTA finds the same.
-template <typename At, typename Found>
-__device__ __forceinline__ void select_find(SelectShared& s, unsigned long long target, unsigned long long above, At bucket_at, Found found) {
-    const int pa = 2 * threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned long long m0 = pa < kSelectBuckets ? s.merged[bucket_at(pa)] : 0ull;
-    const unsigned long long m1 = pa + 1 < kSelectBuckets ? s.merged[bucket_at(pa + 1)] : 0ull;
-    const unsigned long long mine = m0 + m1;
-    unsigned long long incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) s.wsum[warp] = incl;
-    __syncthreads();
-    unsigned long long w = lane < warp ? s.wsum[lane] : 0ull;   // the sums of the warps before this one
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    const unsigned long long need = target - above, excl = w + incl - mine;
-    if (excl < need && need <= excl + mine) {       // the range holds at least `need`, and need >= 1
-        const bool first = excl + m0 >= need;
-        const int b = bucket_at(first ? pa : pa + 1);
-        s.digit = b;
-        s.above = above + excl + (first ? 0ull : m0);
-        found(b, first ? m0 : m1);
-    }
-    __syncthreads();
-}
-// monotone in the logit: two roundings and a clamp
-__device__ __forceinline__ int linear_bucket(float z, float mx, float per_unit) {
-    return (int)fminf(fmaxf((mx - z) * per_unit, 0.f), (float)(kSelectBuckets - 1));
-}
-// The nucleus threshold's key where the deciding bucket holds more tokens than the list takes: their one key, or a radix select
-// over their range of keys, 11 bits at a time from the top, on the same histograms.  z, e: the CTA's slice of n_local tokens.
-// A function of its own, not inlined: few rows need it, and inside the kernel its code costs the others 1 to 2 us of 30.
-__device__ __noinline__ unsigned int select_by_radix(SelectShared& s, const float* __restrict__ z, const double* e, int n_local) {
-    const int deciding = (int)s.digit;
-    const float mx = s.mx, per_unit = s.per_unit;
-    const unsigned long long light = s.light, target = s.target;
-    unsigned long long above = s.above;             // mass of the keys above the range
-    const int n_round = (n_local + 4 * kSampleThreads - 1) / (4 * kSampleThreads) * (4 * kSampleThreads);
-    auto each = [&](auto f) {                       // f(token, logit); past the end: -1
-        for (int v0 = threadIdx.x; v0 < n_round; v0 += 4 * kSampleThreads) {
-            float z4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) z4[u] = v0 + u * kSampleThreads < n_local ? __ldcg(z + v0 + u * kSampleThreads) : -INFINITY;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) f(v0 + u * kSampleThreads < n_local ? v0 + u * kSampleThreads : -1, z4[u]);
-        }
-    };
-    unsigned int lo = 0xffffffffu, hi = 0u;         // the bucket's range of keys
-    each([&](int v, float zv) {
-        if (v >= 0 && linear_bucket(zv, mx, per_unit) == deciding) {
-            const unsigned int key = order_key(zv);
-            lo = min(lo, key);
-            hi = max(hi, key);
-        }
-    });
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31) < kSampleCtas) {
-        asm volatile("red.shared::cluster.min.u32 [%0], %1;" ::"r"(peer_smem(&s.lo, threadIdx.x & 31)), "r"(lo) : "memory");
-        asm volatile("red.shared::cluster.max.u32 [%0], %1;" ::"r"(peer_smem(&s.hi, threadIdx.x & 31)), "r"(hi) : "memory");
-    }
-    cluster_sync_all();                             // the row's range, in every CTA
-    lo = s.lo;
-    unsigned int span = s.hi - lo;
-    constexpr int kBits = 11;
-    static_assert(kSelectBuckets == 1 << kBits, "a digit is one of the buckets");
-    for (int shift = max(32 - __clz((int)span) - kBits, 0); span; shift = max(shift - kBits, 0)) {
-        for (int i = threadIdx.x; i < 3 * kSelectBuckets; i += kSampleThreads) s.hist[0][i] = 0u;
-        __syncthreads();
-        each([&](int v, float zv) {
-            const unsigned int d = order_key(zv) - lo;
-            const int b = v >= 0 && d <= span && linear_bucket(zv, mx, per_unit) == deciding ? (int)(d >> shift) : -1;
-            if (!__any_sync(0xffffffffu, b >= 0)) return;
-            const unsigned long long q = b >= 0 ? sample_mass(e[v]) : 0ull;
-            select_add(s, q >= light ? b : -1, q);
-        });
-        select_merge(s, (int)blockIdx.y);
-        select_find(s, target, above, [](int p) { return kSelectBuckets - 1 - p; }, [](int, unsigned long long) {});
-        above = s.above;
-        const unsigned int at = s.digit << shift;
-        lo += at;
-        span = shift ? min(span - at, (1u << shift) - 1u) : 0u;
-    }
-    cluster_sync_all();                             // every CTA is done with the select's memory
-    return lo;
-}
-
-// NT = tokens per thread: warp w holds the cells w, w + 32, ... of its CTA's slice, four tokens of a cell per lane
-// kNucleus: top_p < 1 (an instance of its own, whose registers the plain one does not pay for)
-template <int NT, bool kNucleus>
-__global__ void __launch_bounds__(kSampleThreads, NT == 32 ? 1 : 0) k_sample(SampleArgs a) {
-    pdl_trigger();
-    pdl_wait();
-    // distributed shared memory may be touched only once every CTA of the cluster has started: awaited before the first use
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    constexpr bool kInSmem = NT * kSampleThreads * kSampleCtas <= kSampleSmemVocab;
-    extern __shared__ __align__(16) double s_e[];       // [tokens of the slice], if kInSmem
-    __shared__ __align__(8) SelectShared s_sel;
-    double* const s_cell = s_sel.cell;
-    // the first CTA's list of the tokens of the deciding bucket lies over its histogram, once that has been merged
-    unsigned int* s_list_key = &s_sel.hist[0][0];
-    unsigned long long* s_list_q = reinterpret_cast<unsigned long long*>(&s_sel.hist[1][0]);
-    static_assert(kSampleListMax <= kSelectBuckets && 2 * kSampleListMax <= kSelectBuckets, "the list does not fit");
-    __shared__ unsigned long long s_slice_q[kSampleCtas];
-    __shared__ double s_warp[32], s_walk_run, s_walk_target;
-    __shared__ float s_slice_max[kSampleCtas], s_slice_min[kSampleCtas], s_maxw[32];
-    __shared__ unsigned int s_count, s_kstar, s_found, s_many;
-    __shared__ int s_last, s_walk_cell;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int V = a.V, row = blockIdx.x, rank = blockIdx.y;   // cluster = (1, 8, 1): rank in the cluster = blockIdx.y
-    const float* __restrict__ z = a.logits + (size_t)row * V;
-    const int n_cells = (V + kSampleCell - 1) / kSampleCell;
-    const int cells_per = (n_cells + kSampleCtas - 1) / kSampleCtas;
-    const int c_lo = min(rank * cells_per, n_cells), c_hi = min(c_lo + cells_per, n_cells);
-    const int v_lo = c_lo * kSampleCell, v_hi = min(c_hi * kSampleCell, V);
-    double* const e = kInSmem ? s_e : a.e + (size_t)row * V + v_lo;   // of token v: e[v - v_lo]
-    auto local = [&](int j) { return ((j >> 2) * 32 + warp) * kSampleCell + (j & 3) * 32 + lane; };   // token j of this thread, in the slice
-    const int n_local = v_hi - v_lo;
-
-    // ---- 1. row maximum, exponentials ----
-    // up to 4 logits per thread stay in registers; more are read again from L2 in every pass, four at a time (16 of them
-    // beside the fp64 exponentials did not fit the 64 registers of a thread)
-    constexpr bool kInRegs = NT <= 4;
-    float zr[kInRegs ? NT : 1];
-    float mx = -INFINITY;
-    auto load_z = [&](int j) { return local(j) < n_local ? __ldcg(z + v_lo + local(j)) : -INFINITY; };
-    if constexpr (kInRegs) {
-#pragma unroll
-        for (int j = 0; j < NT; ++j) zr[j] = load_z(j);
-    }
-    // f(j, logit of token j) for this thread's tokens
-    auto each = [&](auto f) {
-        if constexpr (kInRegs) {
-#pragma unroll
-            for (int j = 0; j < NT; ++j) f(j, zr[j]);
-        } else {
-#pragma unroll 1
-            for (int j0 = 0; j0 < NT; j0 += 4) {
-                float z4[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) z4[u] = load_z(j0 + u);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) f(j0 + u, z4[u]);
-            }
-        }
-    };
-    each([&](int, float zj) { mx = fmaxf(mx, zj); });
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) s_maxw[warp] = mx;
-    if (tid == 0) {   // (with logits that are no numbers nothing may be found: every CTA goes on alike)
-        s_count = 0u; s_kstar = 0u; s_many = 0u;
-        s_sel.digit = 0u; s_sel.above = 0ull; s_sel.lo = 0xffffffffu; s_sel.hi = 0u;
-    }
-    if (kNucleus)
-        for (int i = tid; i < 3 * kSelectBuckets; i += kSampleThreads) s_sel.hist[0][i] = 0u;
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {                                // lane t hands this slice's maximum to the CTA of rank t
-        float sm = s_maxw[lane];
-        for (int o = 16; o > 0; o >>= 1) sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
-        if (lane < kSampleCtas)
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_smem(&s_slice_max[rank], lane)), "f"(sm) : "memory");
-    }
-    cluster_sync_all();
-    mx = s_slice_max[0];
-    for (int i = 1; i < kSampleCtas; ++i) mx = fmaxf(mx, s_slice_max[i]);
-    unsigned long long qsum = 0ull;
-    float low = INFINITY;
-    const bool unit = a.temperature == 1.0;         // x / 1 = x
-    each([&](int j, float zj) {
-        if (local(j) < n_local) {
-            const double x = (double)zj - (double)mx;
-            const double ev = exp(unit ? x : x / a.temperature);
-            e[local(j)] = ev;
-            if (kNucleus) { qsum += sample_mass(ev); low = fminf(low, zj); }
-        }
-    });
-
-    // ---- 2. top-p: key of the smallest logit inside the nucleus (0: every token) ----
-    unsigned int kstar = 0;
-    if constexpr (kNucleus) {
-        for (int o = 16; o > 0; o >>= 1) {
-            qsum += __shfl_xor_sync(0xffffffffu, qsum, o);
-            low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
-        }
-        if (lane == 0) { s_sel.wsum[warp] = qsum; s_maxw[warp] = low; }
-        __syncthreads();                            // also orders this CTA's e stores before other threads' loads below
-        if (warp == 0) {
-            unsigned long long t = s_sel.wsum[lane];
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane < kSampleCtas)
-                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_smem(&s_slice_q[rank], lane)), "l"(t) : "memory");
-        }
-        if (warp == 1) {
-            float t = s_maxw[lane];
-            for (int o = 16; o > 0; o >>= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
-            if (lane < kSampleCtas)
-                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_smem(&s_slice_min[rank], lane)), "f"(t) : "memory");
-        }
-        cluster_sync_all();
-        // One thread works out what the select goes by, the same in every CTA (all of them: their 64-bit divisions queue up).
-        if (tid == 0) {
-            unsigned long long total_q = 0ull;
-            for (int i = 0; i < kSampleCtas; ++i) total_q += s_slice_q[i];
-            const unsigned long long want = (unsigned long long)ceil(a.top_p * (double)total_q);   // mass wanted
-            s_sel.target = want < 1ull ? 1ull : (want > total_q ? total_q : want);
-            // Tokens lighter than (1 - top_p) * total / V weigh less than (1 - top_p) * total together, so the tokens at
-            // or above that weight already hold the mass wanted: the lighter ones lie below the threshold logit and never
-            // decide anything.  They skip the histogram.
-            const unsigned long long least = (unsigned long long)((1.0 - a.top_p) * (double)total_q / (double)V * 0.999999);
-            s_sel.light = least;
-            // buckets linear in the logit: 0 holds the maximum, the last one the minimum or the lightest token that counts, at
-            // exp(-depth) of the maximum: nearly flat rows are spread over all buckets too
-            const float depth = logf(1.0995116e12f / (float)(least > 1ull ? least : 1ull));
-            float mn = s_slice_min[0];
-            for (int i = 1; i < kSampleCtas; ++i) mn = fminf(mn, s_slice_min[i]);
-            const float range = fminf((float)a.temperature * depth, mx - mn);
-            s_sel.mx = mx;
-            s_sel.per_unit = range > 0.f ? (kSelectBuckets - 1) / range : 0.f;
-        }
-        __syncthreads();
-        const unsigned long long light = s_sel.light;
-        const float per_unit = s_sel.per_unit;
-        each([&](int j, float zj) {
-            const unsigned long long q = local(j) < n_local ? sample_mass(e[local(j)]) : 0ull;
-            select_add(s_sel, q >= light && local(j) < n_local ? linear_bucket(zj, mx, per_unit) : -1, q);
-        });
-        select_merge(s_sel, rank);
-        // how many tokens the bucket holds, from its mass and the weight in its middle (the same in every CTA): where they are
-        // far too many for the list, it is not begun
-        select_find(s_sel, s_sel.target, 0ull, [](int p) { return p; }, [&](int b, unsigned long long mass) {
-            const float middle = 1.0995116e12f * (per_unit > 0.f ? expf(-((float)b + 0.5f) / (per_unit * (float)a.temperature)) : 1.f);
-            s_many = (float)mass > 1.5f * kSampleListMax * middle ? 1u : 0u;
-        });
-        const int deciding = (int)s_sel.digit;
-        bool many = s_many;
-        if (!many) {
-            const uint32_t count0 = peer_smem(&s_count, 0), key0 = peer_smem(s_list_key, 0), q0 = peer_smem(s_list_q, 0);
-            each([&](int j, float zj) {
-                if (local(j) < n_local && linear_bucket(zj, mx, per_unit) == deciding) {
-                    const unsigned long long q = sample_mass(e[local(j)]);
-                    if (q >= light && q > 0ull) {
-                        unsigned int at;
-                        asm volatile("atom.shared::cluster.add.u32 %0, [%1], 1;" : "=r"(at) : "r"(count0) : "memory");
-                        if (at < (unsigned int)kSampleListMax) {
-                            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(key0 + 4u * at), "r"(order_key(zj)) : "memory");
-                            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(q0 + 8u * at), "l"(q) : "memory");
-                        }
-                    }
-                }
-            });
-            cluster_sync_all();                     // the first CTA's list is complete
-            if (rank == 0) {
-                const int n = (int)min(s_count, (unsigned int)kSampleListMax);
-                if (tid < n) {                      // the largest key whose upper set holds the mass wanted
-                    const unsigned int key = s_list_key[tid];
-                    unsigned long long mass = s_sel.above;
-                    for (int i = 0; i < n; ++i) mass += s_list_key[i] >= key ? s_list_q[i] : 0ull;
-                    if (mass >= s_sel.target) atomicMax(&s_kstar, key);
-                }
-                __syncthreads();
-                if (tid < kSampleCtas) {
-                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_smem(&s_found, tid)), "r"(s_kstar) : "memory");
-                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_smem(&s_many, tid)), "r"(s_count > (unsigned int)kSampleListMax ? 1u : 0u) : "memory");
-                }
-            }
-            cluster_sync_all();                     // s_found, s_many; every CTA is done with its table of merged masses
-            kstar = s_found;
-            many = s_many;
-        }
-        if (many) kstar = select_by_radix(s_sel, z + v_lo, e, n_local);
-    } else {
-        __syncthreads();                            // this CTA's e stores before other threads' loads below
-    }
-
-    // ---- 3. cell sums of this CTA's slice, into every CTA's table ----
-#pragma unroll(kInRegs ? NT / 4 : 1)
-    for (int j0 = 0; j0 < NT; j0 += 4) {
-        const int c = c_lo + (j0 >> 2) * 32 + warp;
-        if (c < c_hi) {
-            double s = 0.0;
-            float z4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) z4[u] = kInRegs ? zr[kInRegs ? j0 + u : 0] : kNucleus ? load_z(j0 + u) : 0.f;
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (local(j0 + u) < n_local && (!kNucleus || order_key(z4[u]) >= kstar)) s += e[local(j0 + u)];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane < kSampleCtas)
-                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(peer_smem(&s_cell[c], lane)), "l"(__double_as_longlong(s)) : "memory");
-        }
-    }
-    cluster_sync_all();                             // all cell sums are in place, in every CTA
-
-    // exclusive scan of the cell sums in vocabulary order: thread t owns cells [t*per, (t+1)*per)
-    const int per = (n_cells + kSampleThreads - 1) / kSampleThreads;
-    const int c0 = min(tid * per, n_cells), c1 = min(c0 + per, n_cells);
-    double mine = 0.0;
-    for (int c = c0; c < c1; ++c) mine += s_cell[c];
-    double incl = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    double before = 0.0, total = 0.0;
-    for (int i = 0; i < 32; ++i) {
-        if (i < warp) before += s_warp[i];
-        total += s_warp[i];
-    }
-    // [lower, upper] of consecutive threads tile [0, total] exactly: lower is the previous thread's upper, computed by
-    // the same additions, so exactly one thread sees lower < target <= upper
-    double lower = __shfl_up_sync(0xffffffffu, incl, 1);
-    lower = lane == 0 ? before : before + lower;
-    const double upper = before + incl;
-    const double target = sample_uniform(a.seed, a.pos0 + row) * total;
-    if (tid == 0) s_walk_cell = -1;
-    __syncthreads();
-    if (lower < target && target <= upper) {
-        double run = lower;
-        int c = c0;
-        while (c < c1 - 1 && run + s_cell[c] < target) run += s_cell[c++];
-        s_walk_cell = c;
-        s_walk_run = run;
-        s_walk_target = target;
-    }
-    __syncthreads();
-    const int walk_cell = s_walk_cell;              // the same in every CTA; -1: no finite mass (a logit that is no number)
-    if (walk_cell < 0 ? rank != 0 : walk_cell < c_lo || walk_cell >= c_hi) return;   // another CTA's
-    if (walk_cell >= 0 && warp == 0) {
-        // the cell that holds u * total, walked by one warp: lane l sums tokens 4l .. 4l+3 of the cell in order, the lane
-        // sums are scanned in lane order, and the first token whose cumulative mass reaches the target is the sample
-        constexpr int kPerLane = kSampleCell / 32;
-        const int v0 = walk_cell * kSampleCell + lane * kPerLane;
-        const double run0 = s_walk_run, tgt = s_walk_target;
-        double ev[kPerLane];
-#pragma unroll
-        for (int j = 0; j < kPerLane; ++j) {
-            const int v = v0 + j, vc = min(v, V - 1);
-            const double e1 = e[vc - v_lo];
-            const unsigned int kv = kstar ? order_key(__ldcg(z + vc)) : 0xffffffffu;
-            ev[j] = v < V && kv >= kstar ? e1 : 0.0;
-        }
-        double mine4 = 0.0;
-#pragma unroll
-        for (int j = 0; j < kPerLane; ++j) mine4 += ev[j];
-        double incl4 = mine4;
-        for (int o = 1; o < 32; o <<= 1) {
-            const double t = __shfl_up_sync(0xffffffffu, incl4, o);
-            if (lane >= o) incl4 += t;
-        }
-        double acc = run0 + (incl4 - mine4);
-        int hit = -1, last_mass = -1;
-#pragma unroll
-        for (int j = 0; j < kPerLane; ++j) {
-            if (ev[j] > 0.0) last_mass = v0 + j;
-            acc += ev[j];
-            if (hit < 0 && ev[j] > 0.0 && acc >= tgt) hit = v0 + j;
-        }
-        const unsigned int hits = __ballot_sync(0xffffffffu, hit >= 0);
-        const unsigned int masses = __ballot_sync(0xffffffffu, last_mass >= 0);
-        int pick;
-        if (hits) pick = __shfl_sync(0xffffffffu, hit, __ffs(hits) - 1);
-        else if (masses) pick = __shfl_sync(0xffffffffu, last_mass, 31 - __clz(masses));   // the walk fell an ulp short
-        else pick = walk_cell * kSampleCell;
-        if (lane == 0) {
-            a.token[a.r0 + row] = pick;
-            __threadfence();
-        }
-    }
-    if (walk_cell < 0 && tid == 0) {
-        a.token[a.r0 + row] = 0;
-        __threadfence();
-    }
-    if (!a.mirror.host) return;                     // nothing to publish: the completion counter is not touched
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicInc(a.counter, gridDim.x - 1) == gridDim.x - 1;   // one CTA per row, the one that owns the walked cell; wraps back to zero
-        __threadfence();
-    }
-    __syncthreads();
-    if (s_last) publish_results(a.mirror);
-}
-template <int NT, bool kNucleus> static bool launch_sample_nt(cudaStream_t st, const SampleArgs& a, int cells_per) {
-    const size_t smem = NT * kSampleThreads * kSampleCtas <= kSampleSmemVocab ? sizeof(double) * (size_t)cells_per * kSampleCell : 0;
-    static bool configured[kMaxDevices];             // function attributes are per device
-    const int dev = current_device();
-    if (dev < 0) return false;
-    if (!configured[dev]) {
-        if (cudaFuncSetAttribute(k_sample<NT, kNucleus>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) != cudaSuccess) return false;
-        configured[dev] = true;
-    }
-    return launch_kc(k_sample<NT, kNucleus>, dim3(a.m, kSampleCtas), dim3(kSampleThreads), smem, st, kSampleCtas, a) == cudaSuccess;
-}
-template <bool kNucleus> static bool launch_sample_top(cudaStream_t st, const SampleArgs& a) {
-    // the fewest tokens per thread that hold a CTA's slice: 32 warps x NT / 4 cells
-    const int n_cells = (a.V + kSampleCell - 1) / kSampleCell, cells_per = (n_cells + kSampleCtas - 1) / kSampleCtas;
-    if (cells_per <= 32) return launch_sample_nt<4, kNucleus>(st, a, cells_per);
-    if (cells_per <= 64) return launch_sample_nt<8, kNucleus>(st, a, cells_per);
-    if (cells_per <= 128) return launch_sample_nt<16, kNucleus>(st, a, cells_per);
-    return launch_sample_nt<32, kNucleus>(st, a, cells_per);
-}
-bool launch_sample(cudaStream_t st, const SampleArgs& a) {
-    return a.top_p < 1.0 ? launch_sample_top<true>(st, a) : launch_sample_top<false>(st, a);
-}
-
 __global__ void k_init_pages(int* pt, int n) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) pt[i] = i;
