@@ -16,8 +16,8 @@
 namespace sb {
 
 static int g_default_gemm = -1;   // -1: pick tcgen05 for bf16 when available
-static int g_fuse = 3;            // bit 0: SwiGLU in the epilogue of the tcgen05 gate/up GEMM; bit 1: RoPE + append + attention + chunk merge in one launch
-static int g_wide_prefill = 1;    // prefill: up to 128 prompt rows per pass of the weight-streaming GEMMs (bf16, tcgen05 path)
+static int g_fuse = 3;            // bit 0: SwiGLU in the gate/up GEMM (tcgen05: in its epilogue); bit 1: RoPE + append + attention + chunk merge in one launch
+static int g_wide_prefill = 1;    // prefill: up to 512 prompt rows per pass of the weight-streaming GEMMs (bf16, tcgen05 path)
 static int g_qkv_ahead = 1;       // draft loop: issue the next layer step's norm + QKV GEMM while waiting for the exit decision
 static int g_trace = 0;           // 1: the stateless layer call times every launch with CUDA events and prints them
 

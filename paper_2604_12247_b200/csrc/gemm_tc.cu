@@ -349,8 +349,7 @@ __global__ void __launch_bounds__(kTcThreads, NB <= 4 ? 2 : 1) k_tc(const __grid
         }
         if (kHead) {
             // lanes -> warp: butterfly merge (both partners compute the same merged triple), of the rows there are: five
-            // merges with an exponential each per row, at the end of the kernel with nothing left to hide them (all eight rows
-            // for one row's exit test: 50.2 us instead of 47.9)
+            // merges with an exponential each per row, at the end of the kernel with nothing left to hide them
 #pragma unroll
             for (int i = 0; i < kMaxW; ++i) {
                 if (i >= p.r0 && i < p.r0 + p.m) {
@@ -851,11 +850,15 @@ static int choose_pair_half(int n_rows, int G) {
 // busiest cluster spends.  G = clusters.  Measured: a k block costs a cluster 0.34-0.38 us whatever the tile width
 // (N = 112, 160, 176 or 256 columns; at 256 that is the measured tensor peak, and 4 stages instead of 6 cost 5 % only),
 // so narrow tiles buy nothing below ~96 rows per CTA: the cost of an item is charged as if it had at least
-// that many (floor 32 / 64 / 96 / 128: 512-token prefill 22.4 / 20.2 / 20.0 / 20.4 ms).
+// that many (floor 32 / 64 / 96 / 128: 512-token prefill 22.4 / 20.2 / 20.0 / 20.4 ms).  Why a narrow one takes as long is not
+// settled: the tensor pipe's active share falls with N, so it is not the pipe that is busy for the rest.
 // With several tiles of rows every width costs the same (charged as 128 rows): fewest and widest items; floor 96 / 128, us
 // per layer: 7B 512 tokens 383 / 378, Llama-3 shape 437 / 424, 13B 300 tokens 458 / 438.
 static int g_pair_floor_rows = 96, g_pair_split_pm = 30;
 static int pair_floor_rows(int n_tiles) { return n_tiles > 1 ? kTileRows : g_pair_floor_rows; }
+// One more k split of a pass of several tiles writes and reads all its rows once more: 7B output projection, 512 rows, in 2 / 3 /
+// 4 splits 33 / 36 / 41 us, where the balance of the clusters alone would take 4.
+static int pair_split_pm(int n_tiles) { return n_tiles > 1 ? 45 : g_pair_split_pm; }
 // Passes of several tiles: k blocks that one accumulator takes in at most (where the matrix is split at all).  The tensor
 // core truncates as it accumulates, so the error of a sum grows with its length, though the balance would be as good with fewer
 // splits.  Hidden state from its fp64 value, 7B shape, after 512 / 300 prompt rows (6 / 4 seeds): QKV, output and down
@@ -897,7 +900,7 @@ static void choose_split_cta_pair(const int* n_rows, int n_mats, int KB, int G, 
             for (int j = 0; j < n_mats; ++j) chunks += (n_rows[j] + 2 * R - 1) / (2 * R);
             const long long per = (chunks * S * n_tiles + G - 1) / G;
             const double cost = (double)per * (R > pair_floor_rows(n_tiles) ? R : pair_floor_rows(n_tiles)) * ((KB + S - 1) / S) *
-                                (1.0 + 0.001 * g_pair_split_pm * (S - 1));
+                                (1.0 + 0.001 * pair_split_pm(n_tiles) * (S - 1));
             if (cost < best - 1e-9) { best = cost; bR = R; bS = S; }
         }
     *R_out = bR;
@@ -919,7 +922,7 @@ static int choose_cols_cta_pair(int n_rows, int G, int n_tiles = 1) {
 // (multiple of 16, up to 256) so that every cluster has ONE item, in two parts of half the columns, each with an accumulator
 // of its own, which meet the same activation tile: no second round at half fill, and the activations are brought once.
 // 0: the items of choose_cols_cta_pair are the better choice.  (Epilogue and main loop of an item don't overlap then: for a
-// single round only.)  7B, 75 rows: 11008 columns in 2 rounds of 80 columns 57 us, in one of 152 columns 48.
+// single round only.)  7B, 75 rows: 11008 columns in 2 rounds of 96 columns 55 us, in one of 160 columns 47.
 static int choose_one_round_cols(int n_rows, int G, int two_round_cols) {
     const int h = ((n_rows + G - 1) / G + 15) / 16 * 16;
     if (h <= kTileRows || h > 2 * kTileRows) return 0;
